@@ -45,6 +45,11 @@ void bandlu_selftest_div_nz_host(const double *x, const double *d, double *q, in
 int bandlu_selftest_div_device(const double *x, const double *d, double *q, int64_t n, int use_division,
                                cudaStream_t stream);
 
+/* The kernel that gbtrf starts from for a band (n >= 1): 0 the one-warp register window,
+ * 1 the shared-memory window (which needs kl + ku >= 2), 2 the multi-CTA kernel or, where
+ * that cannot be launched, the column-by-column one.  Computed on the host. */
+int bandlu_selftest_gbtrf_path(int64_t n, int kl, int ku, int64_t ldab);
+
 #ifdef __cplusplus
 }
 #endif

@@ -90,6 +90,8 @@ def load():
         lib.bandlu_selftest_div_nz_host.restype = None
         lib.bandlu_selftest_div_device.argtypes = [vp, vp, vp, i64, i32, vp]
         lib.bandlu_selftest_div_device.restype = ctypes.c_int
+        lib.bandlu_selftest_gbtrf_path.argtypes = [i64, i32, i32, i64]
+        lib.bandlu_selftest_gbtrf_path.restype = ctypes.c_int
         lib.bandlu_peak_dfma.argtypes = [vp, i32, i32, i32, i32, vp]
         lib.bandlu_peak_dmma.argtypes = [i32, vp, i32, i32, i32, i32, vp]
         lib.bandlu_peak_hbm_read.argtypes = [vp, i64, vp, i32, vp]
@@ -261,6 +263,11 @@ def bandlu_selftest_div_nz_host(x, d, q, n: int) -> None:
 def bandlu_selftest_div_device(x, d, q, n: int, use_division: int, stream=None) -> int:
     """Self-test hook: the library's known-divisor division (or plain division) on the device."""
     return load().bandlu_selftest_div_device(_ptr(x), _ptr(d), _ptr(q), n, use_division, _stream(stream))
+
+
+def bandlu_selftest_gbtrf_path(n: int, kl: int, ku: int, ldab: int) -> int:
+    """Self-test hook: the kernel gbtrf starts from (0 register window, 1 shared-memory window, 2 wider)."""
+    return load().bandlu_selftest_gbtrf_path(n, kl, ku, ldab)
 
 
 def bandlu_peak_dfma(d_sink, blocks: int, threads: int, chains: int, iters: int, stream=None) -> int:

@@ -129,6 +129,9 @@ int launch_dense_to_band_cm(const double *A, int64_t lda, int64_t n, int kl, int
 // hand-off flags live in stream-ordered scratch).
 int launch_gbtrf(int64_t n, int kl, int ku, double *AB, int64_t ldab, int *ipiv, int *d_info, cudaStream_t s,
                  bool allow_alloc = true);
+// The kernel that launch_gbtrf starts from: 0 the register window, 1 the shared-memory
+// window, 2 the multi-CTA kernel or, where that cannot be launched, the generic one.
+int gbtrf_path(int64_t n, int kl, int ku, int64_t ldab);
 int launch_gbtrf_wide(int64_t n, int kl, int ku, double *AB, int64_t ldab, int *ipiv, int *d_info, cudaStream_t s,
                       bool *used);
 // dispatch_lu_async: the decision and the conversion with (kl, ku) read on the

@@ -223,7 +223,7 @@ __device__ __forceinline__ void window_factor(int n, int kl, int ku, double *__r
     const int rs = min(lane, L - 1);  // a slot to read for the lanes that hold none
     int pos = lane < L ? lane : INT_MAX;
     double cur = W[rs], v1 = W[L + rs];  // columns j, j+1
-    int q1 = 1, q2 = 2;                  // column slots of columns j+1, j+2 (C >= 6)
+    int q1 = 1, q2 = 2;                  // column slots of columns j+1, j+2 (C >= 3: factor_path)
     // the step's pivot: its slot, its offset, an exact zero; the multipliers; U(j, j+1)
     int wl = 0, p = 0;
     bool zp = false;
@@ -506,7 +506,8 @@ __global__ void __launch_bounds__(1024) k_gbtrf_generic(long long n, int kl, int
 // in registers (regwin.cuh).  Fill-row entries above the matrix are cleared
 // first, as the elimination clears every fill row; the window writes the rest.
 // Called by one whole warp.
-__device__ __forceinline__ void regwin_factor(int n, int kl, int ku, double *__restrict__ AB, int ldab,
+template <class Off>
+__device__ __forceinline__ void regwin_factor(int n, int kl, int ku, double *__restrict__ AB, Off ldab,
                                               int *__restrict__ ipiv, int *__restrict__ d_info) {
   const int kv = kl + ku, lane = threadIdx.x & 31;
   if (kl > 0) {
@@ -520,22 +521,30 @@ __device__ __forceinline__ void regwin_factor(int n, int kl, int ku, double *__r
   int *const pvp[1] = {ipiv};
   const int klv[1] = {kl}, kuv[1] = {ku};
   int info[1];
-  regwin::window_gbtrf<1, 1>(abp, ldab, n, klv, kuv, pvp, info);
+  regwin::window_gbtrf<1, 1, Off>(abp, ldab, n, klv, kuv, pvp, info);
   if (lane == 0) *d_info = info[0];
 }
 
-__global__ void __launch_bounds__(32) k_gbtrf_regwin(int n, int kl, int ku, double *__restrict__ AB, int ldab,
+template <class Off>
+__global__ void __launch_bounds__(32) k_gbtrf_regwin(int n, int kl, int ku, double *__restrict__ AB, Off ldab,
                                                      int *__restrict__ ipiv, int *__restrict__ d_info) {
-  regwin_factor(n, kl, ku, AB, ldab, ipiv, d_info);
+  regwin_factor<Off>(n, kl, ku, AB, ldab, ipiv, d_info);
 }
+
+// The register window's 32-bit offsets reach every entry.
+__host__ __device__ inline bool offsets_fit(long long n, long long ldab) { return (n + 1) * ldab < (long long)INT_MAX; }
 
 // The path choice of launch_gbtrf (without the multi-CTA kernel), shared by the
 // host launcher and the device-side dispatch: 0 register window, 1 shared-memory
-// window (*K: its template parameter, *smem: its bytes), 2 generic.
+// window (*K: its template parameter, *smem: its bytes), 2 generic.  Every band with
+// L*C <= 32 takes path 0, whatever its storage, so path 1 has C >= 6 (C >= L); its
+// panel warp requires 3 (columns j+1 and j+2 beside column j, in slots of their own).
+// The windows count rows a few steps past the last one in 32 bits.
 __host__ __device__ inline int factor_path(long long n, int kl, int ku, long long ldab, int *K, size_t *smem) {
   const long long kv = (long long)kl + ku;
-  if ((kl + 1LL) * (kv + 1) <= 32 && (n + 1) * ldab < (long long)INT_MAX) return 0;
-  const long long L = kl + 1, C = kv + 1;
+  const long long L = kl + 1LL, C = kv + 1;
+  if (n > INT_MAX - 64) return 2;
+  if (L * C <= 32) return 0;
   if (kl <= kWinMaxKl && kl + kv + 1 <= 256 && L * (kv - 2) <= kWinMaxTrail) {
     const int k = (int)((L * C + kNUT - 1) / kNUT);
     *smem = (size_t)((2 * L + kEnt) * C) * sizeof(double);
@@ -583,7 +592,10 @@ __global__ void __launch_bounds__(kWinWarps * 32, 1) k_gbtrf_on_device(int n, do
     return;
   }
   if (path == 0) {
-    if (threadIdx.x < 32) regwin_factor(n, kl, ku, AB, (int)ldab, ipiv, d_info);
+    if (threadIdx.x < 32) {
+      if (offsets_fit(n, ldab)) regwin_factor<int>(n, kl, ku, AB, (int)ldab, ipiv, d_info);
+      else regwin_factor<long long>(n, kl, ku, AB, ldab, ipiv, d_info);
+    }
   } else if (path == 1) {
     window_factor_k(K, n, kl, ku, AB, ldab, ipiv, d_info, W, sh);
   } else {
@@ -602,6 +614,12 @@ int launch_window(long long n, int kl, int ku, double *AB, long long ldab, int *
 
 }  // namespace
 
+int gbtrf_path(int64_t n, int kl, int ku, int64_t ldab) {
+  int K = 0;
+  size_t smem = 0;
+  return factor_path(n, kl, ku, ldab, &K, &smem);
+}
+
 int launch_gbtrf(int64_t n, int kl, int ku, double *AB, int64_t ldab, int *ipiv, int *d_info, cudaStream_t s,
                  bool allow_alloc) {
   if (n == 0) {
@@ -612,7 +630,8 @@ int launch_gbtrf(int64_t n, int kl, int ku, double *AB, int64_t ldab, int *ipiv,
   size_t smem = 0;
   const int path = factor_path(n, kl, ku, ldab, &K, &smem);
   if (path == 0) {
-    k_gbtrf_regwin<<<1, 32, 0, s>>>((int)n, kl, ku, AB, (int)ldab, ipiv, d_info);
+    if (offsets_fit(n, ldab)) k_gbtrf_regwin<int><<<1, 32, 0, s>>>((int)n, kl, ku, AB, (int)ldab, ipiv, d_info);
+    else k_gbtrf_regwin<long long><<<1, 32, 0, s>>>((int)n, kl, ku, AB, ldab, ipiv, d_info);
     BANDLU_CHECK_LAUNCH();
     return BANDLU_OK;
   }

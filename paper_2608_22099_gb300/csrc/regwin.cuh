@@ -50,9 +50,9 @@ __host__ __device__ __forceinline__ int planes_of(int kl, int kv, int W) {
 // entry a step writes belongs to a row that entered the window earlier, so reading
 // and writing in place do not collide.  Same operations in the same order as the
 // unblocked elimination: the factors are bit-identical to it.
-// 32-bit offsets: requires (n+1) * ldab < 2^31.
-template <int S, int NR>
-__device__ __forceinline__ void window_gbtrf(double *const (&abs)[S], int ldab, int n, const int (&kls)[S],
+// Off: the type of offsets into AB; int requires (n+1) * ldab < 2^31, long long takes any storage.
+template <int S, int NR, class Off = int>
+__device__ __forceinline__ void window_gbtrf(double *const (&abs)[S], Off ldab, int n, const int (&kls)[S],
                                              const int (&kus)[S], int *const (&ipivs)[S], int (&infos)[S]) {
   static_assert(S == 1 || NR == 1, "several segments or several planes");
   constexpr int W = 32 / S;
@@ -84,14 +84,15 @@ __device__ __forceinline__ void window_gbtrf(double *const (&abs)[S], int ldab, 
     if (pos[k] < n && c < n && c - s <= ku) w[k] = __ldcg(ab + (kv + s - c) + c * ldab);
   }
   // this lane's column in the window: coff columns after j, at ab + cb
-  int coff = c, cb = c * ldab;
+  int coff = c;
+  Off cb = c * ldab;
   int jc = 0;  // column slot of column j
   // q[s] holds the entry of the entering row of the next step j with j % kWinPrefetch == s
   // (row j+1+kl) in this lane's column of that window (columns j+1..j+1+kv); it is refilled
   // kWinPrefetch steps ahead.  The step loop is unrolled by kWinPrefetch so that every slot is
   // one register (rotating the slots would wait on each load a step after issuing it).
   int qoff = c == 0 ? kv : c - 1, qcol = c == 0 ? C : c;  // for the next refill: offset in its window, column
-  int qat = (kv + kl - qoff) + qcol * ldab;
+  Off qat = (kv + kl - qoff) + qcol * ldab;
   double q[kWinPrefetch];
   auto refill = [&](int row) {
     double v = 0.0;
@@ -220,7 +221,7 @@ __device__ __forceinline__ void window_gbtrf(double *const (&abs)[S], int ldab, 
       const bool piv = prow && (NR == 1 || k == kp);
       const int np = pos[k] == j ? j + p : pos[k];
       // U(j, j+coff) -> AB(kv-coff, j+coff); l_{pos, j} -> AB(kv+pos-j, j)
-      const int at = cb + kv + (piv ? -coff : np - j);
+      const Off at = cb + kv + (piv ? -coff : np - j);
       const bool put = piv ? j + coff < n : (head && np < n);
       const double keep = piv ? qs : (head ? 0.0 : w[k]);  // a slot that changes hands, or no update
       const double l = a[k] * rc;                          // multiplier l_{pos, j}

@@ -2,7 +2,7 @@
 // integer-pipe reciprocal used on the pivot chain and the known-divisor division
 // of the back substitution, callable on the host and on the device so tests can
 // compare them bit for bit with IEEE division (and the quotient with its zero test
-// on the host).
+// on the host), and the choice of the factorisation kernel.
 #include "bandlu_selftest.h"
 #include "common.cuh"
 #include "rcp.cuh"
@@ -54,6 +54,10 @@ int bandlu_selftest_div_device(const double *x, const double *d, double *q, int6
   k_divk<<<(unsigned)blocks, 256, 0, stream>>>(x, d, q, n, use_division);
   BANDLU_CHECK_LAUNCH();
   return BANDLU_OK;
+}
+
+int bandlu_selftest_gbtrf_path(int64_t n, int kl, int ku, int64_t ldab) {
+  return bandlu::gbtrf_path(n, kl, ku, ldab);
 }
 
 void bandlu_selftest_rcp_host(const double *x, double *y, int64_t n) {
