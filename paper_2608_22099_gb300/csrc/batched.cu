@@ -229,12 +229,12 @@ __device__ int warp_gbtrf(double *ab, int ldab, int n, int kl, int ku, int *ipiv
 
 // One matrix by one warp with its window in NR registers a lane.
 template <int NR>
-__device__ __forceinline__ int one_window(double *ab, int ldab, int n, int kl, int ku, int *ipiv) {
+__device__ __forceinline__ int one_window(double *ab, unsigned ldab, int n, int kl, int ku, int *ipiv) {
   double *const abp[1] = {ab};
   int *const pvp[1] = {ipiv};
   const int klt[1] = {kl}, kut[1] = {ku};
   int inf[1];
-  regwin::window_gbtrf<1, NR>(abp, ldab, n, klt, kut, pvp, inf);
+  regwin::window_gbtrf<1, NR, unsigned>(abp, ldab, n, klt, kut, pvp, inf);
   return inf[0];
 }
 
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(128) k_batch_factor(long long n, long long bat
     double *const abp[2] = {AB + b0 * strideAB, AB + (b0 + 1) * strideAB};
     int *const pvp[2] = {ipiv + b0 * strideP, ipiv + (b0 + 1) * strideP};
     int info[2];
-    regwin::window_gbtrf<2, 1>(abp, (int)ldab, (int)n, kl, ku, pvp, info);
+    regwin::window_gbtrf<2, 1, unsigned>(abp, (unsigned)ldab, (int)n, kl, ku, pvp, info);
     if (lane == 0) {
       d_info[b0] = info[0];
       d_info[b0 + 1] = info[1];
@@ -283,10 +283,10 @@ __global__ void __launch_bounds__(128) k_batch_factor(long long n, long long bat
   int *pv = ipiv + b * strideP;
   const int np = planes(t, 32);
   int info;
-  if (np == 1) info = one_window<1>(ABb, (int)ldab, (int)n, kl[t], ku[t], pv);
-  else if (np <= 3) info = one_window<3>(ABb, (int)ldab, (int)n, kl[t], ku[t], pv);
-  else if (np <= 5) info = one_window<5>(ABb, (int)ldab, (int)n, kl[t], ku[t], pv);
-  else if (np <= kMaxPlanes) info = one_window<kMaxPlanes>(ABb, (int)ldab, (int)n, kl[t], ku[t], pv);
+  if (np == 1) info = one_window<1>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
+  else if (np <= 3) info = one_window<3>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
+  else if (np <= 5) info = one_window<5>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
+  else if (np <= kMaxPlanes) info = one_window<kMaxPlanes>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
   else info = warp_gbtrf(ABb, (int)ldab, (int)n, kl[t], ku[t], pv);
   if (lane == 0) d_info[b] = info;
 }

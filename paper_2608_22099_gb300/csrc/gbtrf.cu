@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(kWinWarps * 32, 1) k_gbtrf_on_device(int n, do
   }
   if (path == 0) {
     if (threadIdx.x < 32) {
-      if (offsets_fit(n, ldab)) regwin_factor<int>(n, kl, ku, AB, (int)ldab, ipiv, d_info);
+      if (offsets_fit(n, ldab)) regwin_factor<unsigned>(n, kl, ku, AB, (unsigned)ldab, ipiv, d_info);
       else regwin_factor<long long>(n, kl, ku, AB, ldab, ipiv, d_info);
     }
   } else if (path == 1) {
@@ -630,7 +630,7 @@ int launch_gbtrf(int64_t n, int kl, int ku, double *AB, int64_t ldab, int *ipiv,
   size_t smem = 0;
   const int path = factor_path(n, kl, ku, ldab, &K, &smem);
   if (path == 0) {
-    if (offsets_fit(n, ldab)) k_gbtrf_regwin<int><<<1, 32, 0, s>>>((int)n, kl, ku, AB, (int)ldab, ipiv, d_info);
+    if (offsets_fit(n, ldab)) k_gbtrf_regwin<unsigned><<<1, 32, 0, s>>>((int)n, kl, ku, AB, (unsigned)ldab, ipiv, d_info);
     else k_gbtrf_regwin<long long><<<1, 32, 0, s>>>((int)n, kl, ku, AB, ldab, ipiv, d_info);
     BANDLU_CHECK_LAUNCH();
     return BANDLU_OK;

@@ -50,11 +50,14 @@ __host__ __device__ __forceinline__ int planes_of(int kl, int kv, int W) {
 // entry a step writes belongs to a row that entered the window earlier, so reading
 // and writing in place do not collide.  Same operations in the same order as the
 // unblocked elimination: the factors are bit-identical to it.
-// Off: the type of offsets into AB; int requires (n+1) * ldab < 2^31, long long takes any storage.
-template <int S, int NR, class Off = int>
+// Off: the type of offsets into AB; unsigned requires (n+1) * ldab < 2^31, long long takes any
+// storage.  A lane's offsets run on past column n, by up to C + kWinPrefetch columns, to places
+// that nothing reads: a 32-bit type must wrap there, not overflow.
+template <int S, int NR, class Off>
 __device__ __forceinline__ void window_gbtrf(double *const (&abs)[S], Off ldab, int n, const int (&kls)[S],
                                              const int (&kus)[S], int *const (&ipivs)[S], int (&infos)[S]) {
   static_assert(S == 1 || NR == 1, "several segments or several planes");
+  static_assert(sizeof(Off) == 8 || Off(-1) > Off(0), "32-bit offsets wrap");
   constexpr int W = 32 / S;
   const int lane = threadIdx.x & 31;
   const int seg = lane / W, sl = lane - seg * W, base = seg * W;
