@@ -190,6 +190,8 @@ int dispatch_lu_async(const double *A, int64_t n, int64_t lda, double *AB, int64
  *     B(i, c) = fma(-B(j, c), U(i,j), B(i, c)) for i = max(0, j-kl-ku)..j-1.
  * (The zero tests are those of the reference BLAS.)  A singular U (a zero
  * U(j,j)) yields infinities or NaNs, as in LAPACK; callers check info first.
+ * Inside the wide sweeps warps wait for one another with a time limit; should a wait
+ * ever give up, the entries of B that depend on it are NaN.
  * Arguments (all DEVICE pointers): 1 n >= 0, 2 kl >= 0, 3 ku >= 0, 4 nrhs >= 0,
  * 5 AB (read only), 6 ldab >= 2*kl+ku+1, 7 ipiv (1-based, read only),
  * 8 B (COLUMN-major n x nrhs, overwritten with X), 9 ldb >= max(1, n).
@@ -205,6 +207,8 @@ int gbtrs(int64_t n, int kl, int ku, int64_t nrhs, const double *AB, int64_t lda
  * Returns what dispatch_lu returns.  On BANDLU_OK the solve is enqueued on
  * `stream`; it reads *d_info on the device and leaves B as it is when the
  * factor is singular (info > 0), so no further host synchronisation is needed.
+ * *d_info is -BANDLU_ERR_TIMEOUT, with NaN in a column of B, should a wait inside
+ * the solve give up.
  * On BANDLU_NOT_BANDED nothing further is enqueued and B is untouched.
  * Arguments: 1 A, 2 n, 3 lda, 4 B (COLUMN-major n x nrhs), 5 ldb >= max(1, n),
  * 6 nrhs >= 0, 7 AB, 8 ldab >= 1, 9 ipiv, 10 h_kl, 11 h_ku (HOST), 12 d_info.
@@ -225,7 +229,9 @@ int dispatch_solve(const double *A, int64_t n, int64_t lda, double *B, int64_t l
  *   upper, j = n-1..0:  if b_j != 0:  b_j = b_j / A(j,j);  b_i = fma(-b_j, A(i,j), b_i), i = max(0, j-k)..j-1
  * Arguments: 1 lower (1 = lower, 0 = upper triangle), 2 n >= 0, 3 k (0 <= k <=
  * max(0, n-1)), 4 A, 5 lda >= max(1, n), 6 B (COLUMN-major n x nrhs, DEVICE),
- * 7 ldb >= max(1, n), 8 nrhs >= 0, 9 d_info (DEVICE, always written).
+ * 7 ldb >= max(1, n), 8 nrhs >= 0, 9 d_info (DEVICE, always written;
+ * -BANDLU_ERR_TIMEOUT, with NaN in a column of B, should a wait inside the solve
+ * give up).
  * Returns BANDLU_OK, -i for a bad argument i, BANDLU_ERR_CUDA.  Asynchronous.
  * Scratch: none.
  */
@@ -263,7 +269,7 @@ int bandlu_classify(int64_t n, int kl, int ku, int64_t ldab);
  *           skipped on the device when the factor is singular, as in dispatch_solve);
  *   DENSE: nothing is enqueued and B is untouched (the caller's dense LU).
  * *d_info is written by every branch but DENSE (first zero diagonal entry, or
- * gbtrf's info).  *h_kl, *h_ku and *h_kind (HOST) are always written.
+ * gbtrf's info; -BANDLU_ERR_TIMEOUT as in trsv_band and dispatch_solve).  *h_kl, *h_ku and *h_kind (HOST) are always written.
  * Returns BANDLU_OK, BANDLU_NOT_BANDED (the DENSE branch), -i for a bad
  * argument i, or an error code.
  * Arguments: 1 A, 2 n, 3 lda, 4 B (COLUMN-major n x nrhs), 5 ldb >= max(1, n),

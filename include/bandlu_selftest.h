@@ -50,6 +50,15 @@ int bandlu_selftest_div_device(const double *x, const double *d, double *q, int6
  * that cannot be launched, the column-by-column one.  Computed on the host. */
 int bandlu_selftest_gbtrf_path(int64_t n, int kl, int ku, int64_t ldab);
 
+/* One CTA-wide sweep of gbtrs over one right-hand side b (DEVICE, n doubles, in place) with
+ * factors AB, ipiv of gbtrf (33 <= kl <= 128, kl + ku <= 160), in which something never arrives:
+ * what = 0 the forward sweep, the copy of column `lost` of the multipliers; 1 the forward sweep,
+ * the value of step `lost`; 2 the backward sweep, the value of step `lost`.  lost < 0: nothing is
+ * lost.  A wait in the sweep then gives up after about a second, the entries of b formed from what
+ * never came are NaN and *d_info (DEVICE) is -BANDLU_ERR_TIMEOUT.  Returns 0, -1 (what), -3 (n, kl, ku or ldab) or BANDLU_ERR_CUDA. */
+int bandlu_selftest_sweep_lost(int what, int lost, int n, int kl, int ku, const double *AB, int ldab,
+                               const int *ipiv, double *b, int *d_info, cudaStream_t stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -92,6 +92,8 @@ def load():
         lib.bandlu_selftest_div_device.restype = ctypes.c_int
         lib.bandlu_selftest_gbtrf_path.argtypes = [i64, i32, i32, i64]
         lib.bandlu_selftest_gbtrf_path.restype = ctypes.c_int
+        lib.bandlu_selftest_sweep_lost.argtypes = [i32, i32, i32, i32, i32, vp, i32, vp, vp, vp, vp]
+        lib.bandlu_selftest_sweep_lost.restype = ctypes.c_int
         lib.bandlu_peak_dfma.argtypes = [vp, i32, i32, i32, i32, vp]
         lib.bandlu_peak_dmma.argtypes = [i32, vp, i32, i32, i32, i32, vp]
         lib.bandlu_peak_hbm_read.argtypes = [vp, i64, vp, i32, vp]
@@ -268,6 +270,13 @@ def bandlu_selftest_div_device(x, d, q, n: int, use_division: int, stream=None) 
 def bandlu_selftest_gbtrf_path(n: int, kl: int, ku: int, ldab: int) -> int:
     """Self-test hook: the kernel gbtrf starts from (0 register window, 1 shared-memory window, 2 wider)."""
     return load().bandlu_selftest_gbtrf_path(n, kl, ku, ldab)
+
+
+def bandlu_selftest_sweep_lost(what: int, lost: int, n: int, kl: int, ku: int, AB, ldab: int, ipiv, b, d_info,
+                               stream=None) -> int:
+    """Self-test hook: a CTA-wide sweep of gbtrs in which the value (or column) of step `lost` never arrives."""
+    return load().bandlu_selftest_sweep_lost(what, lost, n, kl, ku, _ptr(AB), ldab, _ptr(ipiv), _ptr(b),
+                                             _ptr(d_info), _stream(stream))
 
 
 def bandlu_peak_dfma(d_sink, blocks: int, threads: int, chains: int, iters: int, stream=None) -> int:

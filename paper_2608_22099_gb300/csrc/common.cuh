@@ -160,9 +160,10 @@ struct WideDeferred {
 int prepare_gbtrf_wide_deferred(int64_t n, int64_t ldab, cudaStream_t s, WideDeferred *wd);
 int launch_gbtrf_wide_deferred(const WideDeferred &wd, int64_t n, double *AB, int64_t ldab, int *ipiv,
                                const int *d_kl, const int *d_ku, int *d_info, cudaStream_t s);
-// d_info: when not null and *d_info != 0 (a singular factor), B is left as it is.
+// d_info: when not null and *d_info != 0 (a singular factor), B is left as it is.  When a wait of a
+// sweep gives up, its right-hand side ends in NaN and *d_info (where not null) is -BANDLU_ERR_TIMEOUT.
 int launch_gbtrs(int64_t n, int kl, int ku, int64_t nrhs, const double *AB, int64_t ldab, const int *ipiv, double *B,
-                 int64_t ldb, const int *d_info, cudaStream_t s);
+                 int64_t ldb, int *d_info, cudaStream_t s);
 // Triangular solve with the band of width k of A's lower (or upper) triangle,
 // and the diagonal solve; both write *d_info (first zero diagonal entry).
 int launch_trsv(bool lower, int64_t n, int k, const double *A, int64_t lda, double *B, int64_t ldb, int64_t nrhs,

@@ -161,28 +161,28 @@ constexpr int kRingPf = 8;  // steps the backward sweep reads ahead
 template <int MAXT, bool kStaged>
 __global__ void __launch_bounds__(MAXT, 1)
     k_gbtrs_block_fwd(int n, int kl, int ku, const double *__restrict__ AB, int ldab, const int *__restrict__ ipiv,
-                      double *__restrict__ B, long long ldb, const int *__restrict__ d_info) {
+                      double *__restrict__ B, long long ldb, int *__restrict__ d_info) {
   extern __shared__ __align__(16) double columns[];
   __shared__ trwin::Ring ring;
   __shared__ trwin::BlockShared bs;
   __shared__ unsigned long long full[2];
   if (d_info != nullptr && *d_info != 0) return;  // a singular factor: B is left as it is
   trwin::block_sweep_piv<kStaged>(B + (long long)blockIdx.x * ldb, n, kl, trwin::GbLower{AB, ldab, kl + ku}, ipiv,
-                                  ring, trwin::Stage{columns, trwin::stage_pitch(kl), full}, bs);
+                                  ring, trwin::Stage{columns, trwin::stage_pitch(kl), full}, bs, d_info);
 }
 
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT) k_gbtrs_ring_bwd(int n, int kl, int ku, const double *__restrict__ AB, int ldab,
                                                          double *__restrict__ B, long long ldb,
-                                                         const int *__restrict__ d_info) {
+                                                         int *__restrict__ d_info) {
   __shared__ trwin::Ring ring;
   if (d_info != nullptr && *d_info != 0) return;
   const int kv = kl + ku;
-  trwin::ring_sweep_div<kRingPf, false>(B + (long long)blockIdx.x * ldb, n, kv, trwin::GbUpper{AB, ldab, kv, n}, ring);
+  trwin::ring_sweep_div<kRingPf, false>(B + (long long)blockIdx.x * ldb, n, kv, trwin::GbUpper{AB, ldab, kv, n}, ring, d_info);
 }
 
 int launch_block_fwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, const int *ipiv, double *B,
-                     long long ldb, const int *d_info, cudaStream_t s) {
+                     long long ldb, int *d_info, cudaStream_t s) {
   const int nt = trwin::block_threads(kl);
   if (kl <= trwin::kStageWidth) {
     // (n = 4096, kl = ku = 100, both sweeps: 335 ns a row staged, 374 from memory)
@@ -200,7 +200,7 @@ int launch_block_fwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab
 }
 
 int launch_ring_bwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, double *B, long long ldb,
-                     const int *d_info, cudaStream_t s) {
+                     int *d_info, cudaStream_t s) {
   const int nt = trwin::ring_threads_div(kl + ku);
   if (nt <= 512)
     k_gbtrs_ring_bwd<512><<<(unsigned)nrhs, nt, 0, s>>>(n, kl, ku, AB, ldab, B, ldb, d_info);
@@ -214,7 +214,7 @@ constexpr int kOneWarpPf = 16;  // steps a one-warp sweep reads ahead: they must
 
 template <int RW>
 void launch_fwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, const int *ipiv, double *B, long long ldb,
-                const int *d_info, cudaStream_t s) {
+                int *d_info, cudaStream_t s) {
   const int wpb = 4;
   k_gbtrs_fwd<RW, kOneWarpPf><<<(unsigned)((nrhs + wpb - 1) / wpb), 32 * wpb, 0, s>>>(n, kl, ku, nrhs, AB, ldab,
                                                                                       ipiv, B, ldb, d_info);
@@ -222,7 +222,7 @@ void launch_fwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, con
 
 template <int RW>
 void launch_bwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, double *B, long long ldb,
-                const int *d_info, cudaStream_t s) {
+                int *d_info, cudaStream_t s) {
   const int wpb = 4;
   k_gbtrs_bwd<RW, kOneWarpPf><<<(unsigned)((nrhs + wpb - 1) / wpb), 32 * wpb, 0, s>>>(n, kl, ku, nrhs, AB, ldab,
                                                                                       B, ldb, d_info);
@@ -234,7 +234,7 @@ void launch_bwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, dou
 constexpr int kOneWarp = 64;
 
 int launch_sweeps(int n, int kl, int ku, int nrhs, const double *AB, int ldab, const int *ipiv, double *B,
-                  long long ldb, const int *d_info, cudaStream_t s) {
+                  long long ldb, int *d_info, cudaStream_t s) {
   if (kl > 0 && n > 1) {
     const int wf = kl + 1;
     if (wf > kOneWarp) {
@@ -257,7 +257,7 @@ int launch_sweeps(int n, int kl, int ku, int nrhs, const double *AB, int ldab, c
 }  // namespace
 
 int launch_gbtrs(int64_t n, int kl, int ku, int64_t nrhs, const double *AB, int64_t ldab, const int *ipiv, double *B,
-                 int64_t ldb, const int *d_info, cudaStream_t s) {
+                 int64_t ldb, int *d_info, cudaStream_t s) {
   if (n == 0 || nrhs == 0) return BANDLU_OK;
   const long long win = (long long)kl + ku + 1;  // rows the backward window needs (>= kl + 1)
   if (n <= INT_MAX / 2 && ldab <= INT_MAX && nrhs <= INT_MAX) {

@@ -2,10 +2,12 @@
 // integer-pipe reciprocal used on the pivot chain and the known-divisor division
 // of the back substitution, callable on the host and on the device so tests can
 // compare them bit for bit with IEEE division (and the quotient with its zero test
-// on the host), and the choice of the factorisation kernel.
+// on the host), the choice of the factorisation kernel, and the solve's CTA sweeps with
+// a value that never arrives.
 #include "bandlu_selftest.h"
 #include "common.cuh"
 #include "rcp.cuh"
+#include "trwin.cuh"
 
 namespace {
 __global__ void k_rcp(const double *__restrict__ x, double *__restrict__ y, long long n) {
@@ -26,9 +28,49 @@ __global__ void k_divk(const double *__restrict__ x, const double *__restrict__ 
     }
   }
 }
+
+// The sweeps' hand-over with the value (or the copied column) of one step lost.
+struct LossyRing : bandlu::trwin::Ring {
+  int lost;
+  __device__ __forceinline__ void put(int k, double v, bool c) { bandlu::trwin::Ring::put(k, v, c && k != lost); }
+};
+struct LossyStage : bandlu::trwin::Stage {
+  int lost;
+  __device__ __forceinline__ void copy(int k, const double *from, unsigned bytes, unsigned bar) const {
+    if (k != lost) bandlu::trwin::Stage::copy(k, from, bytes, bar);
+  }
+};
+
+__global__ void __launch_bounds__(256) k_sweep_lost(int what, int lost, int n, int kl, int ku, const double *AB,
+                                                    int ldab, const int *ipiv, double *b, int *d_info) {
+  extern __shared__ __align__(16) double columns[];
+  __shared__ LossyRing ring;
+  __shared__ bandlu::trwin::BlockShared bs;
+  __shared__ unsigned long long full[2];
+  const int kv = kl + ku;
+  if (threadIdx.x == 0) ring.lost = what == 0 ? -1 : lost;
+  if (what == 2) {
+    bandlu::trwin::ring_sweep_div<8, false>(b, n, kv, bandlu::trwin::GbUpper{AB, ldab, kv, n}, ring, d_info);
+  } else {
+    const LossyStage st{{columns, bandlu::trwin::stage_pitch(kl), full}, what == 0 ? lost : -1};
+    bandlu::trwin::block_sweep_piv<true>(b, n, kl, bandlu::trwin::GbLower{AB, ldab, kv}, ipiv, ring, st, bs, d_info);
+  }
+}
 }  // namespace
 
 extern "C" {
+
+int bandlu_selftest_sweep_lost(int what, int lost, int n, int kl, int ku, const double *AB, int ldab, const int *ipiv,
+                               double *b, int *d_info, cudaStream_t stream) {
+  if (what < 0 || what > 2) return -1;
+  if (n < 1 || kl < 33 || kl > 128 || ku < 0 || kl + ku > 160 || ldab < 2 * kl + ku + 1) return -3;
+  const int threads = what == 2 ? bandlu::trwin::ring_threads_div(kl + ku) : bandlu::trwin::block_threads(kl);
+  const size_t smem = 64 * (size_t)bandlu::trwin::stage_pitch(kl) * sizeof(double);
+  if (!bandlu::allow_dynamic_smem(reinterpret_cast<const void *>(k_sweep_lost), (int)smem)) return BANDLU_ERR_CUDA;
+  k_sweep_lost<<<1, threads, smem, stream>>>(what, lost, n, kl, ku, AB, ldab, ipiv, b, d_info);
+  BANDLU_CHECK_LAUNCH();
+  return BANDLU_OK;
+}
 
 void bandlu_selftest_div_host(const double *x, const double *d, double *q, int64_t n) {
   for (int64_t i = 0; i < n; ++i) {

@@ -59,14 +59,14 @@ __global__ void __launch_bounds__(128) k_trsv_window(int n, int k, const double 
 template <int MAXT, bool kLower>
 __global__ void __launch_bounds__(MAXT) k_trsv_ring(int n, int k, const double *__restrict__ A, long long lda,
                                                     double *__restrict__ B, long long ldb,
-                                                    const int *__restrict__ d_info) {
+                                                    int *__restrict__ d_info) {
   __shared__ trwin::Ring ring;
   if (*d_info != 0) return;
   double *b = B + (long long)blockIdx.x * ldb;
   if (kLower)
-    trwin::ring_sweep_div<8, true>(b, n, k, trwin::DenseLower{A, lda}, ring);
+    trwin::ring_sweep_div<8, true>(b, n, k, trwin::DenseLower{A, lda}, ring, d_info);
   else
-    trwin::ring_sweep_div<8, false>(b, n, k, trwin::DenseUpper{A, lda, n}, ring);
+    trwin::ring_sweep_div<8, false>(b, n, k, trwin::DenseUpper{A, lda, n}, ring, d_info);
 }
 
 __global__ void __launch_bounds__(128) k_trsv_generic(int lower, long long n, long long k, const double *__restrict__ A,
@@ -104,7 +104,7 @@ __global__ void k_diag_solve(long long n, const double *__restrict__ A, long lon
 
 template <bool kLower>
 int launch_trsv_window(int n, int k, const double *A, long long lda, double *B, long long ldb, int nrhs,
-                       const int *d_info, cudaStream_t s) {
+                       int *d_info, cudaStream_t s) {
   const int w = k + 1;
   // one warp with two registers a lane was slower than the CTA (n = 4096, k = 40: 262 ns a row, 222)
   if (w > 32) {

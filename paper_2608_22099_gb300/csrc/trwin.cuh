@@ -312,9 +312,9 @@ __device__ __forceinline__ void sweep_piv(double *b, int n, int kw, const Src &s
 // registers a lane), k = 100 178 (542; 218 when a follower polled every step by itself);
 // both sweeps after gbtrf, kl = ku = 100 338 (645 with a CTA-wide window and a barrier per
 // step), 256 433 (1035), 400 521 (1080).
-// A poll gives up after kWaitLimitCycles and raises *giveup, on which every poll of the
-// CTA returns at once (with the empty slot's NaN: the results show it); in a correct run
-// none does.
+// A poll gives up after kWaitLimitCycles, says so in *d_info and raises giveup, on which
+// every wait of the CTA returns at once; what it waited for is then NaN, and so is all that
+// the sweep forms from it.  In a correct run none does.
 constexpr unsigned long long kEmpty = 0xfff8badc0ffee123ull;
 constexpr int kRing = 64;
 // An empty slot, told by its high word alone.
@@ -324,73 +324,70 @@ __device__ __forceinline__ bool slot_empty(unsigned long long v) {
 
 struct Ring {
   alignas(16) unsigned long long x[kRing];
+  int *status;  // *d_info, or null
   int giveup;
-};
 
-// The lane where c holds writes x (predicated: a divergent branch would cost each step more than
-// the store).
-__device__ __forceinline__ void ring_put(Ring &r, int k, double x, bool c) {
-  unsigned long long v = (unsigned long long)__double_as_longlong(x);
-  v = slot_empty(v) ? 0x7fffffffffffffffull : v;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.volatile.shared.u64 [%0], %1;\n\t}" ::"r"(
-                   smem_addr(&r.x[k & (kRing - 1)])),
-               "l"(v), "r"((unsigned)c)
-               : "memory");
-}
-__device__ __forceinline__ unsigned long long ring_peek(Ring &r, int k) {
-  unsigned long long v;
-  asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(v) : "r"(smem_addr(&r.x[k & (kRing - 1)])) : "memory");
-  return v;
-}
-// Polls until get() returns true; on giving up raises *giveup and returns.
-template <class Get>
-__device__ __forceinline__ void ring_poll(Ring &r, Get get) {
-  if (!get()) {
-    long long t0 = 0;
-    for (unsigned it = 1; !get(); ++it) {
-      if ((it & 1023u) == 0) {
-        const long long t = clock64();
-        if (t0 == 0) t0 = t;
-        if (*reinterpret_cast<volatile int *>(&r.giveup) || t - t0 > kWaitLimitCycles) {
-          *reinterpret_cast<volatile int *>(&r.giveup) = 1;
+  __device__ __forceinline__ void init(int *d_info) {  // by the whole CTA, a barrier after it
+    for (int i = threadIdx.x; i < kRing; i += blockDim.x) x[i] = kEmpty;
+    if (threadIdx.x == 0) {
+      status = d_info;
+      giveup = 0;
+    }
+  }
+  __device__ __forceinline__ bool gave_up() const { return *reinterpret_cast<const volatile int *>(&giveup) != 0; }
+  // The lane where c holds writes v (predicated: a divergent branch would cost each step more than
+  // the store).
+  __device__ __forceinline__ void put(int k, double v, bool c) {
+    unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    u = slot_empty(u) ? 0x7fffffffffffffffull : u;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q st.volatile.shared.u64 [%0], %1;\n\t}" ::"r"(
+                     smem_addr(&x[k & (kRing - 1)])),
+                 "l"(u), "r"((unsigned)c)
+                 : "memory");
+  }
+  __device__ __forceinline__ double peek(int k) {
+    unsigned long long v;
+    asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(v) : "r"(smem_addr(&x[k & (kRing - 1)])) : "memory");
+    return __longlong_as_double((long long)v);
+  }
+  // Polls until get() returns true; false when that does not come about.
+  template <class Get>
+  __device__ __forceinline__ bool poll(Get get) {
+    bool ok = get();
+    if (!ok) {
+      const long long t0 = clock64();
+      for (unsigned it = 0; !(ok = get()); ++it) {
+        if ((it & 1023u) == 0 && (gave_up() || clock64() - t0 > kWaitLimitCycles)) {
+          *reinterpret_cast<volatile int *>(&giveup) = 1;
+          if (status != nullptr) *status = -BANDLU_ERR_TIMEOUT;
           break;
         }
       }
     }
+    __syncwarp();
+    return ok;
   }
-  __syncwarp();
-}
-// x of step k, polled by a whole warp (an empty slot's NaN when a poll gave up).
-__device__ __forceinline__ double ring_get(Ring &r, int k) {
-  unsigned long long v = 0;
-  ring_poll(r, [&] {
-    v = ring_peek(r, k);
-    return !slot_empty(v);
-  });
-  return __longlong_as_double((long long)v);
-}
-// x of steps k..k+3, k a multiple of 4.
-__device__ __forceinline__ void ring_get4(Ring &r, int k, double (&x)[4]) {
-  unsigned long long v[4];
-  const unsigned a = smem_addr(&r.x[k & (kRing - 1)]);
-  ring_poll(r, [&] {
-    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(a) : "memory");
-    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[2]), "=l"(v[3]) : "r"(a + 16u) : "memory");
-    return !(slot_empty(v[0]) || slot_empty(v[1]) || slot_empty(v[2]) || slot_empty(v[3]));
-  });
+  // x of steps k..k+3, k a multiple of 4, polled by a whole warp (an empty slot's NaN when the
+  // poll gave up).
+  __device__ __forceinline__ void get4(int k, double (&out)[4]) {
+    unsigned long long v[4];
+    const unsigned a = smem_addr(&x[k & (kRing - 1)]);
+    auto get = [&] {
+      asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(a) : "memory");
+      asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[2]), "=l"(v[3]) : "r"(a + 16u) : "memory");
+      return !(slot_empty(v[0]) || slot_empty(v[1]) || slot_empty(v[2]) || slot_empty(v[3]));
+    };
+    poll(get);
 #pragma unroll
-  for (int s = 0; s < 4; ++s) x[s] = __longlong_as_double((long long)v[s]);
-}
-__device__ __forceinline__ void ring_init(Ring &r) {  // by the whole CTA, a barrier after it
-  for (int i = threadIdx.x; i < kRing; i += blockDim.x) r.x[i] = kEmpty;
-  if (threadIdx.x == 0) r.giveup = 0;
-}
-__device__ __forceinline__ void ring_empty_slot(Ring &r, int k) {
-  asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(smem_addr(&r.x[k & (kRing - 1)])), "l"(kEmpty) : "memory");
-}
-__device__ __forceinline__ void ring_empty(Ring &r, int B) {  // by one warp: the slots of block B
-  ring_empty_slot(r, 32 * B + (threadIdx.x & 31));
-}
+    for (int s = 0; s < 4; ++s) out[s] = __longlong_as_double((long long)v[s]);
+  }
+  __device__ __forceinline__ void empty(int B) {  // by one warp: the slots of block B
+    asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(
+                     smem_addr(&x[(32 * B + (threadIdx.x & 31)) & (kRing - 1)])),
+                 "l"(kEmpty)
+                 : "memory");
+  }
+};
 
 // Threads of a CTA-wide sweep with update width kw <= kRingMax.
 constexpr int kRingMax = 992;  // 1024 threads hold kw + 32 positions
@@ -400,12 +397,12 @@ constexpr int ring_threads_div(int kw) { return kw < 1 ? 64 : (kw + 63) / 32 * 3
 // then c + NW, ...: the chunk of block B is led by its warp, in which the chain of the
 // block stays (quotient, shuffle, multiply-add, as in sweep_div); the other warps follow
 // from the ring, as far behind as they like within the block.
-template <int kPf, bool kFwd, class Src>
-__device__ __forceinline__ void ring_sweep_div(double *b, int n, int kw, const Src &src, Ring &ring) {
+template <int kPf, bool kFwd, class Src, class Ring>
+__device__ __forceinline__ void ring_sweep_div(double *b, int n, int kw, const Src &src, Ring &ring, int *d_info) {
   static_assert(32 % kPf == 0 && kPf % 4 == 0, "blocks of 32 steps, polled by fours");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   auto row = [&](int m) { return kFwd ? m : n - 1 - m; };
-  ring_init(ring);
+  ring.init(d_info);
   int c = warp;   // this warp's chunk
   int cf_c = c;   // the chunk of the next coefficients asked for
   auto pos = [&](int chunk) { return 32 * chunk + lane; };
@@ -424,7 +421,7 @@ __device__ __forceinline__ void ring_sweep_div(double *b, int n, int kw, const S
   for (int s = 0; s < kPf; ++s) fill(s, s);
   __syncthreads();
   for (int kb = 0, B = 0; kb < n; kb += 32, ++B) {
-    if (warp == nw - 1 && B >= 1) ring_empty(ring, B - 1);
+    if (warp == nw - 1 && B >= 1) ring.empty(B - 1);
     if (c == B) {
       double out = 0.0;
       for (int k0 = kb; k0 < kb + 32; k0 += kPf) {
@@ -443,7 +440,7 @@ __device__ __forceinline__ void ring_sweep_div(double *b, int n, int kw, const S
           }
           const int t = lane - o;
           const double u = fma(-cf[s], x, w);
-          ring_put(ring, k, x, lane == o);
+          ring.put(k, x, lane == o);
           out = lane == o ? x : out;
           w = (go && t >= 1 && t <= min(kw, n - 1 - k)) ? u : w;
           fill(s, k + kPf);
@@ -464,7 +461,7 @@ __device__ __forceinline__ void ring_sweep_div(double *b, int n, int kw, const S
           // some position within reach of one of the four steps (none is past the end)
           if (32 * c - k4 - 3 <= kw && 32 * c < n) {  // uniform
             double x[4];
-            ring_get4(ring, k4, x);
+            ring.get4(k4, x);
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
               const int k = k4 + s, t = pos(c) - k;
@@ -495,6 +492,13 @@ struct Stage {
   int pitch;                 // even
   unsigned long long *full;  // [2]: block B's columns have landed, phase B / 2
   __device__ __forceinline__ double *col(int k) const { return buf + (k & 63) * pitch; }
+  // column k's copy, on the barrier of its block
+  __device__ __forceinline__ void copy(int k, const double *from, unsigned bytes, unsigned bar) const {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_addr(col(k))),
+                 "l"(from), "r"(bytes), "r"(bar)
+                 : "memory");
+  }
 };
 constexpr int stage_pitch(int entries) { return (entries + 3) & ~1; }
 
@@ -503,6 +507,7 @@ __device__ __forceinline__ int stage_off(const double *first) {
   return (int)((reinterpret_cast<unsigned long long>(first) >> 3) & 1ull);
 }
 // By one warp: `len` entries from `first` (this lane's column; len 0 or less: none) for block B.
+template <class Stage>
 __device__ __forceinline__ void stage_block(const Stage &st, int B, int k, const double *first, int len) {
   const int lane = threadIdx.x & 31;
   const int off = stage_off(first);
@@ -513,14 +518,11 @@ __device__ __forceinline__ void stage_block(const Stage &st, int B, int k, const
   if (lane == 0)
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(total) : "memory");
   __syncwarp();
-  if (bytes != 0u)
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(st.col(k))),
-                 "l"(first - off), "r"(bytes), "r"(bar)
-                 : "memory");
+  if (bytes != 0u) st.copy(k, first - off, bytes, bar);
 }
-__device__ __forceinline__ void stage_wait(const Stage &st, int B, Ring &ring) {
-  mbar_wait_warp(st.full + (B & 1), (unsigned)(B >> 1) & 1u, &ring.giveup);
+// Block B's columns have landed; false: they never did.
+__device__ __forceinline__ bool stage_wait(const Stage &st, int B, Ring &ring) {
+  return ring.poll([&] { return mbar_try_wait(st.full + (B & 1), (unsigned)(B >> 1) & 1u); });
 }
 
 // sweep_piv by a CTA, the chain of a block of 32 steps in one warp: the interchanges of a block
@@ -546,9 +548,9 @@ struct BlockShared {
 
 // kStaged: the multipliers through shared memory (kw <= kStageWidth, where the buffers fit), else
 // from memory a group of four steps ahead.
-template <bool kStaged>
+template <bool kStaged, class Ring, class Stage>
 __device__ __forceinline__ void block_sweep_piv(double *b, int n, int kw, const GbLower &src, const int *ipiv,
-                                                Ring &ring, const Stage &st, BlockShared &bs) {
+                                                Ring &ring, const Stage &st, BlockShared &bs, int *d_info) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const bool keeper = warp == nw - 1;
   auto ask_swap = [&](int B) { return __ldg(ipiv + min(32 * B + lane, n - 1)); };
@@ -576,7 +578,7 @@ __device__ __forceinline__ void block_sweep_piv(double *b, int n, int kw, const 
     }
     __syncwarp();
   };
-  ring_init(ring);
+  ring.init(d_info);
   if (kStaged && threadIdx.x == 0) {
     mbar_init(st.full, 1);
     mbar_init(st.full + 1, 1);
@@ -602,9 +604,10 @@ __device__ __forceinline__ void block_sweep_piv(double *b, int n, int kw, const 
   for (int kb = 0, B = 0; kb < n; kb += 32, ++B) {
     if (keeper) {
       if (B >= 1) {
-        b[kb - 32 + lane] = __longlong_as_double((long long)ring_peek(ring, kb - 32 + lane));
-        ring_empty(ring, B - 1);
-        if (kStaged && kb + 32 < n) stage(B + 1);
+        b[kb - 32 + lane] = ring.peek(kb - 32 + lane);
+        ring.empty(B - 1);
+        // (no arrival on a barrier whose phase has never completed: that is a fault)
+        if (kStaged && kb + 32 < n && !__any_sync(FULL, ring.gave_up())) stage(B + 1);
       }
       put_new(B + 1, in);
       in = ask_new(B + 2);
@@ -620,7 +623,7 @@ __device__ __forceinline__ void block_sweep_piv(double *b, int n, int kw, const 
       const int o0 = has ? bs.from[B & 1][at] : 0;
       int pos = kb + o0;
       double w = has ? bs.val[B & 1][pos % kValRing] : 0.0;
-      if (kStaged) stage_wait(st, B, ring);
+      if (kStaged && !stage_wait(st, B, ring)) w = __longlong_as_double(0x7fffffffffffffffll);  // all of the block
       double cf[4];
       unsigned in4 = 0;
       const int a0 = stage_off(src.at(0, 1));
@@ -659,12 +662,12 @@ __device__ __forceinline__ void block_sweep_piv(double *b, int n, int kw, const 
             const int o = (k0 + s) & 31;
             const double x = __shfl_sync(FULL, w, o);
             const double u = fma(-c4[s], x, w);
-            ring_put(ring, k0 + s, w, lane == o);
+            ring.put(k0 + s, w, lane == o);
             w = (((m4 >> s) & 1u) && nz(x)) ? u : w;
           }
         } else if (__any_sync(FULL, m4 != 0u)) {
           double x[4];
-          ring_get4(ring, k0, x);  // (the leader writes all four, past the last position too)
+          ring.get4(k0, x);  // (the leader writes all four, past the last position too)
 #pragma unroll
           for (int s = 0; s < 4; ++s) {
             const double u = fma(-c4[s], x[s], w);
@@ -677,7 +680,7 @@ __device__ __forceinline__ void block_sweep_piv(double *b, int n, int kw, const 
     __syncthreads();
   }
   const int last = (n - 1) / 32 * 32 + threadIdx.x;
-  if (threadIdx.x < 32 && last < n) b[last] = __longlong_as_double((long long)ring_peek(ring, last));
+  if (threadIdx.x < 32 && last < n) b[last] = ring.peek(last);
 }
 
 }  // namespace trwin

@@ -51,3 +51,30 @@ def test_trsv_window_edges(n, k, lower):
     got, ginfo = trsv_gpu(A, lower, k, B)
     assert ginfo == info == 0
     assert_same_solution(got, ref)
+
+
+@pytest.mark.parametrize("what,lost", [(0, -1), (0, 40), (1, 5), (1, 199), (2, 70)])
+def test_a_value_that_never_arrives_shows_in_the_result(what, lost):
+    """A CTA-wide sweep in which a copied column (0: forward) or the value of a step (1: forward, 2:
+    backward) is lost: the waits give up after about a second, every entry formed from it is NaN and the
+    status says why."""
+    import torch
+
+    from gpu_helpers import DEV
+    from paper_2608_22099_gb300 import bandlu
+    n, kl, ku = 240, 90, 40
+    A = banded(n, kl, ku, seed=3, dist="normal").numpy() + 100.0 * np.eye(n)  # (no interchanges)
+    ABf, ipiv, _, _ = oracle.gbtrf(oracle.dense_to_band(A, kl, ku), kl, ku)
+    AB, ip = torch.from_numpy(ABf).to(DEV), torch.from_numpy(ipiv).to(DEV)
+    b = torch.ones(n, dtype=torch.float64, device=DEV)
+    info = torch.zeros(1, dtype=torch.int32, device=DEV)
+    assert bandlu.bandlu_selftest_sweep_lost(what, lost, n, kl, ku, AB, ABf.shape[1], ip, b, info) == 0
+    torch.cuda.synchronize()
+    if lost < 0:
+        assert int(info.item()) == 0 and not bool(torch.isnan(b).any())
+    else:
+        assert int(info.item()) == -bandlu.BANDLU_ERR_TIMEOUT
+        # every entry outside the lost step's block takes its multiple; the columns of a block land together
+        first = {0: lost // 32 * 32, 1: lost // 32 * 32 + 32, 2: lost // 32 * 32 + 32}[what]
+        affected = b[first:] if what < 2 else b.flip(0)[first:]
+        assert affected.numel() and bool(torch.isnan(affected).all())
