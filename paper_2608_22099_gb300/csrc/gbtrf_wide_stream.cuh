@@ -49,8 +49,13 @@
 // overwrite those of panel p-(NS+1), which every streamer has read before A can hold
 // block p (each streamer has passed block p on, after reading panel p-NS); a block goes
 // into a streamer's slot once the slot's previous block (SL before) has arrived whole at
-// the next CTA down, which tells the warp that fills the slot (credit).  Every wait is
-// bounded.
+// the next CTA down, which tells the warp that fills the slot (credit).  The slot's readers
+// on the CTA itself have then taken the block: its sender passed it on, and its group sent
+// the band that panel b-r changed.  A block b < r has no such panel and goes on without the
+// group, which must not miss it either (it waits by parity: two blocks later in the slot look
+// like none): on streamers 1..NS-1 the group opens every block's phase itself, and the last
+// streamer's loader waits for its group's word beside the credit (kFreeArrivals).  Every
+// wait is bounded.
 // What paces it: A's column steps (n = 8000, kl = 37, ku = 53: 2.2 of 2.4 us a panel,
 // kl = ku = 256 3.1 of 3.3), once the way of a block round to A -- update CTA, loader, the
 // streamers, each a move and four steps -- takes no longer than NS + 1 panels.  ns a
@@ -96,6 +101,7 @@ struct Chain {
   static constexpr int kRecDepth = NS + 1;  // panels of step records per streamer
   static constexpr int kSlots = SL;         // block slots per streamer
   static constexpr int kHand = NS + 1;      // update CTAs hand block b over after panel b-kHand
+  static constexpr int kFreeArrivals = 2;   // on a slot of the last streamer: the credit, its group
 };
 
 // Whether whole warps of the group can lie beyond the panel's rows: those skip the multiply-adds
@@ -123,7 +129,8 @@ struct StreamShared {
   unsigned long long mb_in[kSlots];            // streamer: block b in slot (b-1) % kSlots, event (b-1) / kSlots
   unsigned long long mb_cred[kSlots];          // streamer: the slot of block b on the CTA it fills is free again
                                                // (block b has arrived further down), event (b-1) / kSlots
-  unsigned long long mb_ldc[kSlots];           // last streamer: the same for its own slots (loader)
+  unsigned long long mb_ldc[kSlots];           // last streamer: the same for its own slots (loader), and its
+                                               // group has been through block b
   unsigned long long mb_blk[kRing];            // A: block b >= 1 arrived (1 arrival + bytes), event b-1
   unsigned long long mb_afree[kAfRing];        // streamer 1: A's buffer of block p stored (A's storer), event p
   unsigned long long mb_pub[kRing];            // A: panel p published (publisher), event p
@@ -502,7 +509,7 @@ __global__ void __launch_bounds__(32 * (CW + 2), 1)
       mbar_init(&ss.mb_in[i], 1);
       mbar_init(&ss.mb_dst[i], 1);
       mbar_init(&ss.mb_cred[i], 1);
-      mbar_init(&ss.mb_ldc[i], 1);
+      mbar_init(&ss.mb_ldc[i], Chain<NS, SL>::kFreeArrivals);
     }
     sh.info = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -689,6 +696,7 @@ __global__ void __launch_bounds__(32 * (CW + 2), 1)
           }
           TR_STAMP(r <= 2 && tid == 0, r, q, 4);
         }
+        if (r == kStreamers && tid == 0) mbar_arrive(&ss.mb_ldc[slot]);
       }
     } else if (warp == sender) {
       // ---------------- sender: the rows panel b-r leaves unchanged, as soon as they can go ----------------
@@ -804,7 +812,7 @@ __global__ void __launch_bounds__(32 * (CW + 2), 1)
     } else if (warp == kCW && r == kStreamers) {
       // ---------------- last streamer, loader: blocks b >= 1 into its slots ----------------
       for (int b = 1; b < g.npan; ++b) {
-        // the slot held block b-kSlots, which has arrived at the next CTA
+        // the slot held block b-kSlots, which has arrived at the next CTA and been through the group
         if (b - kSlots >= 1) {
           unsigned long long *mb = &ss.mb_ldc[(b - 1) % kSlots];
           const unsigned par = ring_parity(b - kSlots - 1, kSlots);
