@@ -138,26 +138,40 @@ __global__ void __launch_bounds__(512) k_detect_flat(const double *__restrict__ 
 // Rows with little padding on any address: the matrix as one run of elements, padding and
 // all, in 16-byte vectors from the first aligned one on (element head + 2f in vector f), in
 // equal chunks.  The run ends with the matrix's last element; a last element without a pair
-// and, on an odd address, the first one are read alone.
+// and, on an odd address, the first one are read alone.  A thread's row and column are
+// carried along: its vectors are a fixed distance apart, so a division a thread is enough
+// (with one for every nonzero element a dense matrix of n = 16383 took 607 us, 480 element by
+// element; n = 8000, lda = 8006 158, 101 by row segments).  lda < 2^30.
 template <int U>
 __global__ void __launch_bounds__(512) k_detect_run(const double *__restrict__ A, long long n, long long lda,
                                                     long long chunk, int *d_kl, int *d_ku) {
   const long long total = (n - 1) * lda + n;
   const int head = (int)(reinterpret_cast<uintptr_t>(A) >> 3) & 1;
   const long long V = (total - head) / 2;
-  const long long f0 = (long long)blockIdx.x * chunk, f1 = min(V, f0 + chunk);
+  const long long f0 = (long long)blockIdx.x * chunk + threadIdx.x, f1 = min(V, (blockIdx.x + 1) * chunk);
   const ulonglong2 *base = reinterpret_cast<const ulonglong2 *>(A + head);
-  const unsigned long long *el = reinterpret_cast<const unsigned long long *>(A);
-  const long long step = (long long)blockDim.x * U;
-  int lmax = 0, umax = 0;
-  auto see = [&](long long e) {
-    const long long i = e / lda, j = e - i * lda;
-    if (j < n) {
-      lmax = max(lmax, (int)(i - j));
-      umax = max(umax, (int)(j - i));
+  const int cols = (int)n, ld = (int)lda;
+  // (row, column) of this thread's first vector of the pass, and from vector to vector and pass to pass
+  int i = 0, j = 0, di[U + 1], dj[U + 1];
+  if (f0 < f1) {
+    const long long e0 = head + 2 * f0;
+    i = (int)(e0 / lda);
+    j = (int)(e0 - i * lda);
+  }
+#pragma unroll
+  for (int u = 0; u <= U; ++u) {
+    const unsigned d = 2u * u * blockDim.x;
+    di[u] = (int)(d / (unsigned)ld);
+    dj[u] = (int)(d % (unsigned)ld);
+  }
+  int dmax = 0, dmin = 0;  // of row - column over the nonzeros
+  auto see = [&](int r, int c) {
+    if (c < cols) {
+      dmax = max(dmax, r - c);
+      dmin = min(dmin, r - c);
     }
   };
-  for (long long f = f0 + threadIdx.x; f < f1; f += step) {
+  for (long long f = f0; f < f1; f += (long long)blockDim.x * U) {
     ulonglong2 x[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -167,17 +181,29 @@ __global__ void __launch_bounds__(512) k_detect_run(const double *__restrict__ A
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (((x[u].x << 1) | (x[u].y << 1)) != 0ull) {  // rare in a banded matrix
-        const long long e = head + 2 * (f + (long long)u * blockDim.x);
-        if (nz_bits(x[u].x)) see(e);
-        if (nz_bits(x[u].y)) see(e + 1);
+        int r = i + di[u], c = j + dj[u];
+        if (c >= ld) {
+          c -= ld;
+          ++r;
+        }
+        if (nz_bits(x[u].x)) see(r, c);
+        const bool next = c + 1 == ld;
+        if (nz_bits(x[u].y)) see(next ? r + 1 : r, next ? 0 : c + 1);
       }
+    }
+    i += di[U];
+    j += dj[U];
+    if (j >= ld) {
+      j -= ld;
+      ++i;
     }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (head != 0 && nz_bits(__ldcs(el))) see(0);
-    if (((total - head) & 1) != 0 && nz_bits(__ldcs(el + total - 1))) see(total - 1);
+    const unsigned long long *el = reinterpret_cast<const unsigned long long *>(A);
+    if (head != 0 && nz_bits(__ldcs(el))) see(0, 0);
+    if (((total - head) & 1) != 0 && nz_bits(__ldcs(el + total - 1))) see(cols - 1, cols - 1);
   }
-  block_fold(lmax, umax, d_kl, d_ku);
+  block_fold(dmax, -dmin, d_kl, d_ku);
 }
 
 // Clears the outputs; the detection kernel behind it may start at once.
@@ -235,9 +261,11 @@ int launch_detect(const double *A, int64_t n, int64_t lda, int *d_kl, int *d_ku,
   const int sms = device_sms();
   const bool vec = ((reinterpret_cast<uintptr_t>(A) & 15u) == 0) && (lda % 2 == 0);
   cudaError_t e;
-  if (lda - n <= 2 + n / 64 && !(vec && lda == 2 * ((n + 1) / 2))) {
-    // little padding (its bytes are read too): one run of vectors (n = 16383: 343 us, 494 element by
-    // element; n = 8000, lda = 8006: 96 us, 106 by row segments)
+  if (lda - n <= 2 + n / 64 && lda < (1ll << 30) && !(vec && (lda == 2 * ((n + 1) / 2) || n < 4500))) {
+    // little padding (its bytes are read too): one run of vectors, us banded / dense (n = 16383: 308 / 314,
+    // 484 / 482 element by element; n = 8000, lda = 8006: 90 / 86, 98 / 101 by row segments; n = 5000, lda =
+    // 5002: 45 / 43, 50 / 55).  Smaller aligned rows go by segments (n = 4096, lda = 4098: 34 / 35, as one
+    // run 35 / 35; n = 2000, lda = 2002: 18 / 18, 19 / 20).
     const long long V = ((n - 1) * lda + n) / 2 + 1;
     const bool big = V >= (1ll << 20);
     const long long G0 = (long long)sms * (big ? 4 : 8);

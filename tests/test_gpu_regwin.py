@@ -95,3 +95,20 @@ def test_detect_reads_one_run_of_any_alignment(n, pad, off):
         assert bandlu.detect_bandwidth(P.data_ptr() + 8 * off, n, lda, out, out.data_ptr() + 4) == 0
         torch.cuda.synchronize()
         assert out.tolist() == [max(0, i - j), max(0, j - i)], (i, j)
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("n,pad", [(2, 0), (5, 1), (33, 0), (100, 3), (513, 0), (1001, 0), (1500, 9), (4501, 1), (4600, 2)])
+def test_detect_of_matrices_full_of_nonzeros(n, pad, off):
+    """Every row and column that a thread carries along is one of a nonzero: a dense matrix, its triangles,
+    and bands whose edge runs through every vector."""
+    lda = n + pad
+    P = torch.full((n * lda + off,), float("nan"), dtype=torch.float64, device=DEV)
+    M = P[off:].view(n, lda)[:, :n]
+    ones = torch.ones((n, n), dtype=torch.float64, device=DEV)
+    for kl, ku in ((n - 1, n - 1), (0, n - 1), (n - 1, 0), (n // 3, n // 2), (n // 2, 1), (0, 0)):
+        M.copy_(torch.triu(torch.tril(ones, ku), -kl))
+        out = torch.full((2,), -7, dtype=torch.int32, device=DEV)
+        assert bandlu.detect_bandwidth(P.data_ptr() + 8 * off, n, lda, out, out.data_ptr() + 4) == 0
+        torch.cuda.synchronize()
+        assert out.tolist() == [kl, ku]
