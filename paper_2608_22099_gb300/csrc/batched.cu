@@ -9,13 +9,13 @@
 //    from the matrix it has just scanned, which is still in L2).
 //  * k_batch_factor: one warp per matrix, or per pair of matrices where both
 //    windows fit 16 lanes, in place on their band storage, in the xGBTRF order of
-//    operations.  Bands whose active window fits up to kMaxPlanes registers a lane
-//    are factored with the window in registers (window_gbtrf): no shared memory, one
-//    argmax, a few shuffles, and a DMUL and a DFMA per plane and column; wider bands
-//    column by column through memory (warp_gbtrf).  One matrix's chain of columns
-//    bounds it: 500 matrices of n = 201, kl = ku = 5 take 130 us (three planes;
-//    column by column they took 619), 4096 of n = 256, kl = ku = 2 take 136 us (201
-//    with the windows kept in order).
+//    operations.  Bands whose active window fits a register a lane, or, in batches
+//    of few warps, up to nine (takes_window), are factored with the window in registers
+//    (window_gbtrf): no shared memory, one argmax, a few shuffles, and a DMUL and a
+//    DFMA per plane and column; the others column by column through memory
+//    (warp_gbtrf).  One matrix's chain of columns bounds it: 500 matrices of n = 201,
+//    kl = ku = 5 take 130 us (three planes; column by column they took 619), 4096 of n =
+//    256, kl = ku = 2 take 136 us (201 with the windows kept in order).
 //  The band storage written by the first kernel (58.7 MB for 4096 matrices of
 //  n = 256, kl = ku = 2) stays in L2 for the second.  (A single kernel with
 //  scanner and factor warps side by side was slower: the factor warps' loads
@@ -238,18 +238,44 @@ __device__ __forceinline__ int one_window(double *ab, unsigned ldab, int n, int 
   return inf[0];
 }
 
+// Whether a band of np planes goes to a register window, in a batch of `load` warps to each of
+// the chip's sub-partitions (at most kPlanesLoad, all resident with the 128 registers of nine
+// planes).  A window's instructions grow with its planes (1, 3, 5 or 9: each count adds to the
+// kernel, and the counts between cost what the next one does), those of a column through memory
+// with its kl*kv updates, and more warps hide its latencies.  us a call with windows of up to
+// nine planes / column by column (n = 128: 600 and 1200 matrices; n = 64: 1800 and 2400):
+//   kl, ku        600          1200         1800         2400
+//   4, 4          105 / 161    137 / 185     88 / 110    108 / 117     3 planes
+//   6, 6          142 / 206    186 / 233    128 / 133    161 / 143     4
+//   7, 7          143 / 244    191 / 275    130 / 151    163 / 161     4
+//   4, 27         149 / 374    215 / 410    133 / 202    175 / 211     5
+//   10, 5         218 / 284    285 / 315    201 / 169    261 / 182     6
+//   5, 20         219 / 320    295 / 363    205 / 186    264 / 200     6
+//   8, 8          219 / 225    289 / 259    206 / 144    263 / 157     9
+//   8, 23         225 / 525    317 / 572    210 / 277    270 / 297     9
+// Beyond kPlanesLoad column by column is faster for any of them (4096 of n = 64: kl = ku = 4 182
+// with planes, 147 without, 8, 23 475, 352; 20000: 764, 639 and 2044, 1582), in the kernel of one
+// plane, whose 72 registers keep seven warps a sub-partition resident.
+constexpr int kPlanesLoad = 4;
+__device__ __forceinline__ bool takes_window(int np, int load, int kl, int ku) {
+  if (np <= 3) return true;
+  if (np > 9) return false;
+  const int work = kl * (kl + ku);
+  if (np <= 5) return load <= 3 || work >= 100;
+  return load <= 2 || work >= 200;
+}
+
 // Warp b of the first half of the grid takes matrices 2b and 2b+1 together, in
 // 16-lane windows, when both bands fit one; otherwise it takes matrix 2b and its
 // counterpart in the second half (which leaves at once in the first case) takes
-// matrix 2b+1: in a window of up to kMaxPlanes registers a lane, or column by
-// column for wider bands.
-// (The line at nine planes: every band up to kl = 8 with kl+ku+1 <= 32 columns.)
-constexpr int kMaxPlanes = 9;
+// matrix 2b+1: in a register window, of one plane or (kPlanes) of up to nine, or
+// column by column.
+template <bool kPlanes>
 __global__ void __launch_bounds__(128) k_batch_factor(long long n, long long batch, double *__restrict__ AB,
                                                       long long ldab, long long strideAB, int *__restrict__ ipiv,
                                                       long long strideP, const int *__restrict__ d_kl,
                                                       const int *__restrict__ d_ku, int *__restrict__ d_info,
-                                                      const int *__restrict__ d_status, int win_ok) {
+                                                      const int *__restrict__ d_status, int win_ok, int load) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   const long long half = gridDim.x >> 1;
   const bool second = blockIdx.x >= half;
@@ -283,11 +309,15 @@ __global__ void __launch_bounds__(128) k_batch_factor(long long n, long long bat
   int *pv = ipiv + b * strideP;
   const int np = planes(t, 32);
   int info;
-  if (np == 1) info = one_window<1>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
-  else if (np <= 3) info = one_window<3>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
-  else if (np <= 5) info = one_window<5>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
-  else if (np <= kMaxPlanes) info = one_window<kMaxPlanes>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
-  else info = warp_gbtrf(ABb, (int)ldab, (int)n, kl[t], ku[t], pv);
+  if (np == 1) {
+    info = one_window<1>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
+  } else if (kPlanes && takes_window(np, load, kl[t], ku[t])) {
+    if (np <= 3) info = one_window<3>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
+    else if (np <= 5) info = one_window<5>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
+    else info = one_window<9>(ABb, (unsigned)ldab, (int)n, kl[t], ku[t], pv);
+  } else {
+    info = warp_gbtrf(ABb, (int)ldab, (int)n, kl[t], ku[t], pv);
+  }
   if (lane == 0) d_info[b] = info;
 }
 
@@ -315,8 +345,14 @@ int launch_batched(const double *A, int64_t n, int64_t lda, int64_t strideA, int
   const int wpb = 4;
   const long long grid2 = 2 * (((batch + 1) / 2 + wpb - 1) / wpb);  // two warps per pair of matrices
   const int win_ok = (n + 1) * ldab < (int64_t)INT_MAX;  // 32-bit offsets in window_gbtrf
-  k_batch_factor<<<(unsigned)grid2, 32 * wpb, 0, s>>>(n, batch, AB, ldab, strideAB, ipiv, strideP, d_kl, d_ku,
-                                                      d_info, d_status, win_ok);
+  // warps to a sub-partition (every band that storage of up to seven rows admits goes in pairs)
+  const long long subs = 4ll * device_sms(), load = ((ldab <= 7 ? (batch + 1) / 2 : batch) + subs - 1) / subs;
+  if (load <= kPlanesLoad)
+    k_batch_factor<true><<<(unsigned)grid2, 32 * wpb, 0, s>>>(n, batch, AB, ldab, strideAB, ipiv, strideP, d_kl, d_ku,
+                                                              d_info, d_status, win_ok, (int)load);
+  else
+    k_batch_factor<false><<<(unsigned)grid2, 32 * wpb, 0, s>>>(n, batch, AB, ldab, strideAB, ipiv, strideP, d_kl,
+                                                               d_ku, d_info, d_status, win_ok, 0);
   BANDLU_CHECK_LAUNCH();
   return BANDLU_OK;
 }

@@ -55,6 +55,20 @@ def test_single_register_window(n, kl, ku, values):
         assert_parity_with_nan(*gbtrf_gpu(AB, kl, ku), *oracle.gbtrf(AB, kl, ku)[:3])
 
 
+@pytest.mark.parametrize("batch", [600, 1300, 1900, 2500, 5000])
+@pytest.mark.parametrize("kl,ku", [(2, 2), (2, 3), (4, 4), (6, 6), (7, 7), (4, 27), (8, 8), (8, 23), (9, 9)])
+def test_batched_windows_by_the_batch(batch, kl, ku):
+    """The same bands in a window or column by column, as the number of warps on the chip has it: one to
+    four to a sub-partition with up to nine planes, beyond with one."""
+    n, ldab = 35, 2 * kl + ku + 1
+    A = make_dense(n, kl, ku, dist="uniform", seed=batch + kl, batch=batch)
+    got = run_batched(A, ldab)
+    ref = oracle.dispatch_lu_batched(A.numpy(), ldab)
+    for key in ("kl", "ku", "status", "info", "ipiv"):
+        assert np.array_equal(got[key], ref[key]), key
+    assert np.array_equal(got["AB"], ref["AB"])
+
+
 @pytest.mark.parametrize("off", [0, 1])
 @pytest.mark.parametrize("n,pad", [(31, 0), (31, 1), (40, 1), (64, 2), (65, 3), (129, 1), (256, 1)])
 def test_batched_padding_is_not_part_of_the_matrix(n, pad, off):
