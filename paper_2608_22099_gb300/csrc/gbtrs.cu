@@ -12,6 +12,7 @@
 // u_jj uses a reciprocal formed ahead of time (div_quick).  The same operations in
 // the same order as the oracle, so the solution is bit-identical to it.  Interchanges outside j..j+kl (not produced by gbtrf)
 // are ignored.
+#include <algorithm>
 #include <climits>
 
 #include "common.cuh"
@@ -184,12 +185,16 @@ __global__ void __launch_bounds__(MAXT) k_gbtrs_ring_bwd(int n, int kl, int ku, 
 int launch_block_fwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, const int *ipiv, double *B,
                      long long ldb, int *d_info, cudaStream_t s) {
   const int nt = trwin::block_threads(kl);
-  if (kl <= trwin::kStageWidth) {
-    // (n = 4096, kl = ku = 100, both sweeps: 335 ns a row staged, 374 from memory)
+  // Staged while the right-hand sides' CTAs are all on the chip at once: the buffers leave room for
+  // one to three a SM (n = 4096, kl = ku = 100, both sweeps: 335 ns a row staged, 374 from memory; n = 1000,
+  // us staged / from memory: kl = 100, ku = 10, 304 right-hand sides 404 / 431, 456 606 / 490, 4096 4077 /
+  // 3342; kl = ku = 250, 152 416 / 443, 304 814 / 695, 4096 10690 / 9090).
+  const size_t staged = 64 * (size_t)trwin::stage_pitch(kl) * sizeof(double);
+  const size_t own = staged + sizeof(trwin::Ring) + sizeof(trwin::BlockShared) + 2048;  // (and what the driver keeps)
+  if (kl <= trwin::kStageWidth && nrhs <= (long long)device_sms() * std::max<long long>(1, 228 * 1024 / own)) {
     constexpr int most = 64 * trwin::stage_pitch(trwin::kStageWidth) * (int)sizeof(double);
     if (!allow_dynamic_smem(reinterpret_cast<const void *>(k_gbtrs_block_fwd<512, true>), most)) return BANDLU_ERR_CUDA;
-    k_gbtrs_block_fwd<512, true><<<(unsigned)nrhs, nt, 64 * trwin::stage_pitch(kl) * sizeof(double), s>>>(
-        n, kl, ku, AB, ldab, ipiv, B, ldb, d_info);
+    k_gbtrs_block_fwd<512, true><<<(unsigned)nrhs, nt, staged, s>>>(n, kl, ku, AB, ldab, ipiv, B, ldb, d_info);
   } else if (nt <= 512) {
     k_gbtrs_block_fwd<512, false><<<(unsigned)nrhs, nt, 0, s>>>(n, kl, ku, AB, ldab, ipiv, B, ldb, d_info);
   } else {
@@ -210,13 +215,15 @@ int launch_ring_bwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab,
   return BANDLU_OK;
 }
 
-constexpr int kOneWarpPf = 16;  // steps a one-warp sweep reads ahead: they must outlast a DRAM round trip (~2000 clocks)
+// Steps a one-warp sweep reads ahead: they must outlast a DRAM round trip (~2000 clocks).
+template <int RW>
+constexpr int one_warp_pf() { return RW <= 2 ? 16 : 8; }
 
 template <int RW>
 void launch_fwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, const int *ipiv, double *B, long long ldb,
                 int *d_info, cudaStream_t s) {
   const int wpb = 4;
-  k_gbtrs_fwd<RW, kOneWarpPf><<<(unsigned)((nrhs + wpb - 1) / wpb), 32 * wpb, 0, s>>>(n, kl, ku, nrhs, AB, ldab,
+  k_gbtrs_fwd<RW, one_warp_pf<RW>()><<<(unsigned)((nrhs + wpb - 1) / wpb), 32 * wpb, 0, s>>>(n, kl, ku, nrhs, AB, ldab,
                                                                                       ipiv, B, ldb, d_info);
 }
 
@@ -224,7 +231,7 @@ template <int RW>
 void launch_bwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, double *B, long long ldb,
                 int *d_info, cudaStream_t s) {
   const int wpb = 4;
-  k_gbtrs_bwd<RW, kOneWarpPf><<<(unsigned)((nrhs + wpb - 1) / wpb), 32 * wpb, 0, s>>>(n, kl, ku, nrhs, AB, ldab,
+  k_gbtrs_bwd<RW, one_warp_pf<RW>()><<<(unsigned)((nrhs + wpb - 1) / wpb), 32 * wpb, 0, s>>>(n, kl, ku, nrhs, AB, ldab,
                                                                                       B, ldb, d_info);
 }
 
@@ -232,6 +239,11 @@ void launch_bwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab, dou
 // (measured on GB300, n = 4096, ns a row of both sweeps with the line at 64 and at 32 rows: kl =
 // ku = 16 271 / 329, kl = 40, ku = 20 332 / 358, kl = ku = 60, its forward sweep one-warp, 374 / 359).
 constexpr int kOneWarp = 64;
+// With more right-hand sides than sub-partitions the backward sweep stays with one warp up to 128
+// rows: then it is the number of warps that counts (n = 1000, us a call, one warp / CTA: kl = 30, ku = 90, 608
+// right-hand sides 413 / 432, 1024 490 / 744, 16384 4990 / 8230; kl = ku = 40, 456 477 / 421, 800 567 / 564,
+// 4096 1650 / 2120).
+constexpr int kOneWarpMany = 128;
 
 int launch_sweeps(int n, int kl, int ku, int nrhs, const double *AB, int ldab, const int *ipiv, double *B,
                   long long ldb, int *d_info, cudaStream_t s) {
@@ -240,16 +252,18 @@ int launch_sweeps(int n, int kl, int ku, int nrhs, const double *AB, int ldab, c
     if (wf > kOneWarp) {
       const int rc = launch_block_fwd(n, kl, ku, nrhs, AB, ldab, ipiv, B, ldb, d_info, s);
       if (rc != BANDLU_OK) return rc;
-    } else if (wf <= 32) 
+    } else if (wf <= 32)
       launch_fwd<1>(n, kl, ku, nrhs, AB, ldab, ipiv, B, ldb, d_info, s);
     else
       launch_fwd<2>(n, kl, ku, nrhs, AB, ldab, ipiv, B, ldb, d_info, s);
     BANDLU_CHECK_LAUNCH();
   }
   const int wb = kl + ku + 1;
-  if (wb > kOneWarp) return launch_ring_bwd(n, kl, ku, nrhs, AB, ldab, B, ldb, d_info, s);
+  if (wb > (nrhs > 4 * device_sms() ? kOneWarpMany : kOneWarp))
+    return launch_ring_bwd(n, kl, ku, nrhs, AB, ldab, B, ldb, d_info, s);
   if (wb <= 32) launch_bwd<1>(n, kl, ku, nrhs, AB, ldab, B, ldb, d_info, s);
-  else launch_bwd<2>(n, kl, ku, nrhs, AB, ldab, B, ldb, d_info, s);
+  else if (wb <= 64) launch_bwd<2>(n, kl, ku, nrhs, AB, ldab, B, ldb, d_info, s);
+  else launch_bwd<4>(n, kl, ku, nrhs, AB, ldab, B, ldb, d_info, s);
   BANDLU_CHECK_LAUNCH();
   return BANDLU_OK;
 }
