@@ -55,9 +55,10 @@ __global__ void __launch_bounds__(128) k_trsv_window(int n, int k, const double 
     trwin::sweep_div<1, 16, false>(b, n, k, trwin::DenseUpper{A, lda, n});
 }
 
-// Wide triangles: a CTA per right-hand side (trwin.cuh), MAXT its largest size.
-template <int MAXT, bool kLower>
-__global__ void __launch_bounds__(MAXT) k_trsv_ring(int n, int k, const double *__restrict__ A, long long lda,
+// Wide triangles: a CTA per right-hand side (trwin.cuh), MAXT its largest size, MINB of them on an SM
+// (0: as the registers have it).
+template <int MAXT, int MINB, bool kLower>
+__global__ void __launch_bounds__(MAXT, MINB) k_trsv_ring(int n, int k, const double *__restrict__ A, long long lda,
                                                     double *__restrict__ B, long long ldb,
                                                     int *__restrict__ d_info) {
   __shared__ trwin::Ring ring;
@@ -109,10 +110,15 @@ int launch_trsv_window(int n, int k, const double *A, long long lda, double *B, 
   // one warp with two registers a lane was slower than the CTA (n = 4096, k = 40: 262 ns a row, 222)
   if (w > 32) {
     const int nt = trwin::ring_threads_div(k);
+    // CTAs of 17 and 18 warps: two on an SM, with 56 registers, once there are more than SMs (n = 1000, k =
+    // 511, lower, us with 56 / 64 registers: 1 right-hand side 273 / 243, 304 415 / 478, 16384 19950 / 24620,
+    // a warp each took 21830)
     if (nt <= 512)
-      k_trsv_ring<512, kLower><<<(unsigned)nrhs, nt, 0, s>>>(n, k, A, lda, B, ldb, d_info);
+      k_trsv_ring<512, 0, kLower><<<(unsigned)nrhs, nt, 0, s>>>(n, k, A, lda, B, ldb, d_info);
+    else if (nt <= 576 && nrhs > device_sms())
+      k_trsv_ring<576, 2, kLower><<<(unsigned)nrhs, nt, 0, s>>>(n, k, A, lda, B, ldb, d_info);
     else
-      k_trsv_ring<1024, kLower><<<(unsigned)nrhs, nt, 0, s>>>(n, k, A, lda, B, ldb, d_info);
+      k_trsv_ring<1024, 0, kLower><<<(unsigned)nrhs, nt, 0, s>>>(n, k, A, lda, B, ldb, d_info);
     BANDLU_CHECK_LAUNCH();
     return BANDLU_OK;
   }

@@ -78,3 +78,28 @@ def test_a_value_that_never_arrives_shows_in_the_result(what, lost):
         first = {0: lost // 32 * 32, 1: lost // 32 * 32 + 32, 2: lost // 32 * 32 + 32}[what]
         affected = b[first:] if what < 2 else b.flip(0)[first:]
         assert affected.numel() and bool(torch.isnan(affected).all())
+
+
+@pytest.mark.parametrize("kl,ku", [(40, 30), (64, 0), (64, 63), (64, 64), (100, 27), (127, 0), (0, 127), (30, 90), (200, 50),
+                                   (397, 3)])
+@pytest.mark.parametrize("nrhs", [153, 305, 609, 700])
+def test_gbtrs_many_right_hand_sides(kl, ku, nrhs):
+    """More right-hand sides than SMs, than staged CTAs on the chip, and than sub-partitions."""
+    n = 450
+    A = banded(n, kl, ku, seed=kl, dist="normal").numpy()
+    ABf, ipiv, _, _ = oracle.gbtrf(oracle.dense_to_band(A, kl, ku), kl, ku)
+    B = right_hand_sides(n, nrhs, kl + ku)
+    assert_same_solution(gbtrs_gpu(ABf, ipiv, kl, ku, B), oracle.gbtrs(ABf, ipiv, kl, ku, B))
+
+
+@pytest.mark.parametrize("lower", [True, False])
+@pytest.mark.parametrize("k", [100, 480, 481, 512, 513, 544, 545])
+@pytest.mark.parametrize("nrhs", [152, 153, 400])
+def test_trsv_many_right_hand_sides(k, lower, nrhs):
+    n = 1100
+    A = triangle(n, k, lower, seed=k, boost=2.0 + 0.2 * k)
+    B = right_hand_sides(n, nrhs, k)
+    ref, info = oracle.tbsv_dense(A, lower, k, B)
+    got, ginfo = trsv_gpu(A, lower, k, B)
+    assert ginfo == info == 0
+    assert_same_solution(got, ref)
