@@ -6,8 +6,8 @@
  * a * (1/pivot), as DGBTF2 forms them; Sec. III-A names DGBTRF).  These hooks
  * expose that reciprocal so the test suite can check it against the host's and
  * the GPU's own division.  The back substitution of gbtrs divides by the
- * diagonal of U, known before the dividend; it uses a division built on that
- * reciprocal (Markstein's iteration), exposed here for the same check.
+ * diagonal of U, known before the dividend; it multiplies by a 63-bit reciprocal
+ * formed ahead of time, exposed here for the same check.
  */
 #ifndef BANDLU_SELFTEST_H
 #define BANDLU_SELFTEST_H
@@ -28,6 +28,17 @@ void bandlu_selftest_rcp_host(const double *x, double *y, int64_t n);
  * are DEVICE arrays of n doubles; asynchronous on `stream`.
  * Returns 0, -1 (x null), -2 (y null), -3 (n < 0) or BANDLU_ERR_CUDA. */
 int bandlu_selftest_rcp_device(const double *x, double *y, int64_t n, int use_division, cudaStream_t stream);
+
+/* The two straight-line reciprocals by themselves, without the division that takes
+ * the operands they leave: which = 0 the one of the register windows, the
+ * shared-memory window and the chain kernel, 1 the one of the pair and single-CTA
+ * wide kernels.  special[i] = 1 where y[i] is not formed.  HOST (_host) or DEVICE
+ * (_device, asynchronous) arrays of n entries.
+ * _device returns 0, -1 (which), -2..-4 (x, y, special null), -5 (n < 0) or
+ * BANDLU_ERR_CUDA. */
+void bandlu_selftest_rcp_raw_host(int which, const double *x, double *y, int *special, int64_t n);
+int bandlu_selftest_rcp_raw_device(int which, const double *x, double *y, int *special, int64_t n,
+                                   cudaStream_t stream);
 
 /* q[i] = x[i] / d[i] for i < n with the library's known-divisor division, on
  * the host.  x, d and q are HOST arrays of n doubles. */

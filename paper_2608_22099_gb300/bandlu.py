@@ -84,6 +84,10 @@ def load():
         lib.bandlu_selftest_rcp_host.restype = None
         lib.bandlu_selftest_rcp_device.argtypes = [vp, vp, i64, i32, vp]
         lib.bandlu_selftest_rcp_device.restype = ctypes.c_int
+        lib.bandlu_selftest_rcp_raw_host.argtypes = [i32, vp, vp, vp, i64]
+        lib.bandlu_selftest_rcp_raw_host.restype = None
+        lib.bandlu_selftest_rcp_raw_device.argtypes = [i32, vp, vp, vp, i64, vp]
+        lib.bandlu_selftest_rcp_raw_device.restype = ctypes.c_int
         lib.bandlu_selftest_div_host.argtypes = [vp, vp, vp, i64]
         lib.bandlu_selftest_div_host.restype = None
         lib.bandlu_selftest_div_nz_host.argtypes = [vp, vp, vp, i64]
@@ -250,6 +254,16 @@ def bandlu_selftest_rcp_host(x, y, n: int) -> None:
 def bandlu_selftest_rcp_device(x, y, n: int, use_division: int, stream=None) -> int:
     """Self-test hook: the library's reciprocal (or plain division) on the device."""
     return load().bandlu_selftest_rcp_device(_ptr(x), _ptr(y), n, use_division, _stream(stream))
+
+
+def bandlu_selftest_rcp_raw_host(which: int, x, y, special, n: int) -> None:
+    """Self-test hook: a straight-line reciprocal and the operands it leaves (host buffers)."""
+    load().bandlu_selftest_rcp_raw_host(which, _ptr_host(x), _ptr_host(y), _ptr_host(special), n)
+
+
+def bandlu_selftest_rcp_raw_device(which: int, x, y, special, n: int, stream=None) -> int:
+    """Self-test hook: the same on the device."""
+    return load().bandlu_selftest_rcp_raw_device(which, _ptr(x), _ptr(y), _ptr(special), n, _stream(stream))
 
 
 def bandlu_selftest_div_host(x, d, q, n: int) -> None:

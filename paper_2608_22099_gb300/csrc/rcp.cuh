@@ -256,38 +256,18 @@ __host__ __device__ __forceinline__ double div_quick(double x, const Divisor &d,
 __device__ __noinline__ static double div_division(double x, double d) { return x / d; }
 #endif
 
-// x / d given div_known_prep(d).
-__host__ __device__ __forceinline__ double div_known(double x, double d, const Divisor &v) {
-  bool unsure;
-  double q = div_quick(x, v, &unsure);
-  if (unsure) {
+// What the sweeps do with a dividend that div_quick is unsure of: the reference-BLAS
+// zero test (a zero is kept, its sign with it, and not divided; *nonzero false), else
+// the division.  A zero fails div_quick's range test, so it always comes here.  live
+// false: x belongs to no row.
+__host__ __device__ __forceinline__ double div_unsure(double x, double d, bool live, bool *nonzero) {
+  const uint64_t bits = dbits(x);
+  *nonzero = (((uint32_t)(bits >> 32) << 1) | (uint32_t)bits) != 0u;
 #ifdef __CUDA_ARCH__
-    q = div_division(x, d);
+  return *nonzero && live ? div_division(x, d) : x;
 #else
-    q = x / d;
+  return *nonzero && live ? x / d : x;
 #endif
-  }
-  return q;
-}
-
-// The back substitution's quotient with the reference-BLAS zero test: x / d for a
-// nonzero x (div_known), x itself for a zero x (no division, its sign kept).  A
-// zero x fails div_quick's range test and is sorted out in the (rare) fallback.
-__host__ __device__ __forceinline__ double div_known_nz(double x, double d, const Divisor &v) {
-  bool unsure;
-  double q = div_quick(x, v, &unsure);
-  if (unsure) {
-    if (x != 0.0) {
-#ifdef __CUDA_ARCH__
-      q = div_division(x, d);
-#else
-      q = x / d;
-#endif
-    } else {
-      q = x;
-    }
-  }
-  return q;
 }
 
 }  // namespace bandlu

@@ -10,6 +10,30 @@
 #include "trwin.cuh"
 
 namespace {
+// x / d as the sweeps form it, a zero dividend divided like any other.
+__host__ __device__ double quotient(double x, double d) {
+  bool unsure;
+  const double q = bandlu::div_quick(x, bandlu::div_known_prep(d), &unsure);
+  return unsure ? x / d : q;
+}
+// The sweeps' quotient with its zero test.
+double quotient_nz(double x, double d) {
+  bool unsure, nonzero;
+  const double q = bandlu::div_quick(x, bandlu::div_known_prep(d), &unsure);
+  return unsure ? bandlu::div_unsure(x, d, true, &nonzero) : q;
+}
+// A straight-line reciprocal and whether it leaves this operand to the division.
+__host__ __device__ double reciprocal(int which, double x, int *special) {
+  bool s;
+  const double y = which == 0 ? bandlu::rcp_rn_quick(x, &s) : bandlu::rcp_rn_fast(x, &s);
+  *special = s ? 1 : 0;
+  return y;
+}
+__global__ void k_rcp_raw(int which, const double *__restrict__ x, double *__restrict__ y, int *__restrict__ special,
+                          long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    y[i] = reciprocal(which, x[i], special + i);
+}
 __global__ void k_rcp(const double *__restrict__ x, double *__restrict__ y, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = bandlu::rcp_rn(x[i]);
@@ -24,7 +48,7 @@ __global__ void k_divk(const double *__restrict__ x, const double *__restrict__ 
     if (use_division) {
       q[i] = x[i] / d[i];
     } else {
-      q[i] = bandlu::div_known(x[i], d[i], bandlu::div_known_prep(d[i]));
+      q[i] = quotient(x[i], d[i]);
     }
   }
 }
@@ -74,13 +98,13 @@ int bandlu_selftest_sweep_lost(int what, int lost, int n, int kl, int ku, const 
 
 void bandlu_selftest_div_host(const double *x, const double *d, double *q, int64_t n) {
   for (int64_t i = 0; i < n; ++i) {
-    q[i] = bandlu::div_known(x[i], d[i], bandlu::div_known_prep(d[i]));
+    q[i] = quotient(x[i], d[i]);
   }
 }
 
 void bandlu_selftest_div_nz_host(const double *x, const double *d, double *q, int64_t n) {
   for (int64_t i = 0; i < n; ++i) {
-    q[i] = bandlu::div_known_nz(x[i], d[i], bandlu::div_known_prep(d[i]));
+    q[i] = quotient_nz(x[i], d[i]);
   }
 }
 
@@ -104,6 +128,25 @@ int bandlu_selftest_gbtrf_path(int64_t n, int kl, int ku, int64_t ldab) {
 
 void bandlu_selftest_rcp_host(const double *x, double *y, int64_t n) {
   for (int64_t i = 0; i < n; ++i) y[i] = bandlu::rcp_rn(x[i]);
+}
+
+void bandlu_selftest_rcp_raw_host(int which, const double *x, double *y, int *special, int64_t n) {
+  for (int64_t i = 0; i < n; ++i) y[i] = reciprocal(which, x[i], special + i);
+}
+
+int bandlu_selftest_rcp_raw_device(int which, const double *x, double *y, int *special, int64_t n,
+                                   cudaStream_t stream) {
+  if (which < 0 || which > 1) return -1;
+  if (n < 0) return -5;
+  if (n == 0) return BANDLU_OK;
+  if (x == nullptr) return -2;
+  if (y == nullptr) return -3;
+  if (special == nullptr) return -4;
+  long long blocks = (n + 255) / 256;
+  if (blocks > 152ll * 64) blocks = 152ll * 64;
+  k_rcp_raw<<<(unsigned)blocks, 256, 0, stream>>>(which, x, y, special, n);
+  BANDLU_CHECK_LAUNCH();
+  return BANDLU_OK;
 }
 
 int bandlu_selftest_rcp_device(const double *x, double *y, int64_t n, int use_division, cudaStream_t stream) {

@@ -196,8 +196,7 @@ __device__ __forceinline__ void sweep_div(double *b, int n, int kw, const Src &s
         bool go = true;
         if ((__ballot_sync(FULL, unsure) >> o) & 1u) {  // uniform, rare
           const double xo = __shfl_sync(FULL, mine, o), d = __shfl_sync(FULL, bd, o);
-          go = nz(xo);
-          x = go && k < n ? div_division(xo, d) : xo;
+          x = div_unsure(xo, d, k < n, &go);
         }
 #pragma unroll
         for (int r = 0; r < RW; ++r) {
@@ -435,8 +434,7 @@ __device__ __forceinline__ void ring_sweep_div(double *b, int n, int kw, const S
           bool go = true;
           if ((__ballot_sync(FULL, unsure) >> o) & 1u) {  // uniform, rare
             const double xo = __shfl_sync(FULL, w, o), d = __shfl_sync(FULL, bd, o);
-            go = nz(xo);
-            x = go && k < n ? div_division(xo, d) : xo;
+            x = div_unsure(xo, d, k < n, &go);
           }
           const int t = lane - o;
           const double u = fma(-cf[s], x, w);

@@ -63,6 +63,58 @@ def test_reciprocal_device_is_ieee_division(source):
     assert same_bits(y, ref).all(), x[~same_bits(y, ref)][:5]
 
 
+def check_raw_reciprocal(which, x, y, special, ref):
+    """Bit for bit 1/x wherever the operand is not left to the division; what is left: zeros, subnormals,
+    |x| >= 2^1021, infinities and NaN in both, and in which = 0 one quotient in about a thousand, too close
+    to a rounding boundary for its remainder to decide."""
+    left = special != 0
+    bad = ~left & ~same_bits(y, ref)
+    assert not bad.any(), x[bad][:5]
+    expo = (x.view(np.int64) >> 52) & 0x7ff
+    outside = (expo == 0) | (expo >= 2045)
+    assert left[outside].all()
+    if which == 1:
+        assert not left[~outside].any()
+    else:
+        rng = np.random.default_rng(9)
+        plain = ~outside & ((x.view(np.int64) & ((1 << 52) - 1)) != 0)
+        some = rng.permutation(np.nonzero(plain)[0])[:200_000]
+        assert left[some].mean() < 1 / 400
+
+
+@pytest.mark.parametrize("which", [0, 1])
+@pytest.mark.parametrize("source", ["edge", "random"])
+def test_straight_line_reciprocals_host(which, source):
+    x = np.ascontiguousarray(edge_inputs() if source == "edge" else random_inputs(1_000_000, 21))
+    y, special = np.empty_like(x), np.empty(x.size, np.int32)
+    bandlu.bandlu_selftest_rcp_raw_host(which, x, y, special, x.size)
+    with np.errstate(all="ignore"):
+        ref = 1.0 / x
+    if source == "edge":  # (significands next to powers of two: more of them near a boundary)
+        assert not (~(special != 0) & ~same_bits(y, ref)).any()
+    else:
+        check_raw_reciprocal(which, x, y, special, ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("which", [0, 1])
+@pytest.mark.parametrize("source", ["edge", "random"])
+def test_straight_line_reciprocals_device(which, source):
+    import torch
+    x = np.ascontiguousarray(edge_inputs() if source == "edge" else random_inputs(4_000_000, 23))
+    xd = torch.from_numpy(x).cuda()
+    y, special = torch.empty_like(xd), torch.empty(x.size, dtype=torch.int32, device="cuda")
+    assert bandlu.bandlu_selftest_rcp_raw_device(which, xd, y, special, x.size) == 0
+    torch.cuda.synchronize()
+    y, special = y.cpu().numpy(), special.cpu().numpy()
+    with np.errstate(all="ignore"):
+        ref = 1.0 / x
+    if source == "edge":
+        assert not (~(special != 0) & ~same_bits(y, ref)).any()
+    else:
+        check_raw_reciprocal(which, x, y, special, ref)
+
+
 def division_pairs(n, seed):
     """Dividend/divisor pairs: random bit patterns, wide-range normals, equal
     exponents, exact quotients (x = d*m with short m), quotients whose last bits
