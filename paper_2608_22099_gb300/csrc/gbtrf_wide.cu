@@ -1183,8 +1183,8 @@ int chain_group(long long rows) {
   return 13;
 }
 
-// f(std::integral_constant<int, cw>) for a group of chain_group.
-template <class F>
+// f(std::integral_constant<int, cw>) for a group of chain_group, of at most MOST warps.
+template <int MOST, class F>
 int with_chain_group(int cw, F f) {
   switch (cw) {
     case 2: return f(std::integral_constant<int, 2>{});
@@ -1192,11 +1192,22 @@ int with_chain_group(int cw, F f) {
     case 6: return f(std::integral_constant<int, 6>{});
     case 8: return f(std::integral_constant<int, 8>{});
     case 9: return f(std::integral_constant<int, 9>{});
-    case 10: return f(std::integral_constant<int, 10>{});
-    case 12: return f(std::integral_constant<int, 12>{});
-    default: return f(std::integral_constant<int, 13>{});
   }
+  if constexpr (MOST > 9) {
+    switch (cw) {
+      case 10: return f(std::integral_constant<int, 10>{});
+      case 12: return f(std::integral_constant<int, 12>{});
+      case 13: return f(std::integral_constant<int, 13>{});
+    }
+  }
+  return BANDLU_ERR_CUDA;  // (no such group)
 }
+
+// Warps of the device-side dispatch's group, at most.  (Storage for more than 284 subdiagonals is
+// more often one of fewer and of superdiagonals; n = 4000, us a call with the groups of 4 and 9 only / all
+// to 9: kl = ku = 100 3136 / 2845, kl = ku = 150 3215 / 2920, kl = 187, ku = 10 3190 / 2958, kl = ku = 256
+// 3372 / 3378.)
+constexpr int kDeferredMost = 9;
 
 // The chain kernel with NS streamers for one shape: BANDLU_OK, BANDLU_NOT_BANDED when it does not fit
 // or leaves an update CTA more than kChainEach blocks of a panel, BANDLU_ERR_CUDA.
@@ -1305,7 +1316,7 @@ int launch_gbtrf_wide(int64_t n, int kl, int ku, double *AB, int64_t ldab, int *
   int rc = BANDLU_NOT_BANDED;
   // the chain: CTA 0 factors, the streamer CTAs apply the lookahead panels as they stream in
   if (sms >= 4 && !pair_disabled() && !chain_disabled() && rows <= 32 * 13) {
-    rc = with_chain_group(chain_group(rows), [&](auto group) {
+    rc = with_chain_group<13>(chain_group(rows), [&](auto group) {
       return launch_chain_any<decltype(group)::value>(g, sms, span, AB, ipiv, d_info, flags, s);
     });
   }
@@ -1362,11 +1373,8 @@ int prepare_gbtrf_wide_deferred(int64_t n, int64_t ldab, cudaStream_t s, WideDef
   if (!chain_disabled()) {
     // the chain, as in launch_gbtrf_wide
     int gc = 0;
-    // (storage for more than 284 subdiagonals is more often one of fewer and of superdiagonals; n =
-    // 4000, us a call with the groups of 4 and 9 only / all to 9: kl = ku = 100 3136 / 2845, kl =
-    // ku = 150 3215 / 2920, kl = 187, ku = 10 3190 / 2958, kl = ku = 256 3372 / 3378)
-    const int group = chain_group(std::min<long long>(rows_max, 288));
-    const int ns = with_chain_group(group, [&](auto c) {
+    const int group = chain_group(std::min<long long>(rows_max, 32 * kDeferredMost));
+    const int ns = with_chain_group<kDeferredMost>(group, [&](auto c) {
       return chain_fits_any<decltype(c)::value>(ldab, sms, span_max, s, &gc, &smem);
     });
     if (gc < 0) return BANDLU_ERR_CUDA;
@@ -1414,7 +1422,7 @@ int launch_gbtrf_wide_deferred(const WideDeferred &wd, int64_t n, double *AB, in
   g.vec = (reinterpret_cast<uintptr_t>(AB) & 15u) == 0;
   int rc = BANDLU_ERR_CUDA;
   if (wd.chain) {
-    rc = with_chain_group(wd.cw, [&](auto c) {
+    rc = with_chain_group<kDeferredMost>(wd.cw, [&](auto c) {
       return launch_chain_deferred_any<decltype(c)::value>(wd, g, AB, ipiv, d_info, d_kl, d_ku, s);
     });
   } else if (wd.cw == 2) {

@@ -538,11 +538,7 @@ __global__ void __launch_bounds__(32 * (CW + 2), 1)
         rt.send = p + 1 < g.npan;  // streamer 1 applies panel p to block p+1
         TR_STAMP(tid == 0, 0, p, 0);
         factor_panel_stream<CW>(g, buf(p), p, sh, bpar, info, rt, AB, ipiv, ss.lm, ss.cand, p > 0);
-        if (tid == 0) {
-          sh.info = info;
-#pragma unroll
-          for (int k = 0; k < kNB; ++k) sh.pvr[p % kRing][k] = sh.pk[p & 1][k];
-        }
+        if (tid == 0) sh.info = info;
         // the publisher and the storer: each warp arrives once its stores are issued (the
         // arrival releases them); the next panel's reads of lm and sh.pk are ordered by the
         // barrier of the wait for block p+1
