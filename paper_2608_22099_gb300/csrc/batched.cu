@@ -240,8 +240,7 @@ __device__ __forceinline__ int one_window(double *ab, unsigned ldab, int n, int 
 
 // Whether a band of np planes goes to a register window, in a batch of `load` warps to each of
 // the chip's sub-partitions (at most kPlanesLoad, all resident with the 128 registers of nine
-// planes).  A window's instructions grow with its planes (1, 3, 5 or 9: each count adds to the
-// kernel, and the counts between cost what the next one does), those of a column through memory
+// planes).  A window's instructions grow with its planes, those of a column through memory
 // with its kl*kv updates, and more warps hide its latencies.  us a call with windows of up to
 // nine planes / column by column (n = 128: 600 and 1200 matrices; n = 64: 1800 and 2400):
 //   kl, ku        600          1200         1800         2400
@@ -256,6 +255,10 @@ __device__ __forceinline__ int one_window(double *ab, unsigned ldab, int n, int 
 // Beyond kPlanesLoad column by column is faster for any of them (4096 of n = 64: kl = ku = 4 182
 // with planes, 147 without, 8, 23 475, 352; 20000: 764, 639 and 2044, 1582), in the kernel of one
 // plane, whose 72 registers keep seven warps a sub-partition resident.
+// Instantiated are 3, 5 and 9 planes; a count between runs the next one's window.  That costs it up to
+// 22% of a call (600 of n = 128 with a window of its own / the next one's: kl = ku = 4, two planes, 84 / 105
+// us, 6, 6, four, 129 / 141, 5, 20, six, 171 / 219, 7, 24, eight, 207 / 224), and a window each would more
+// than double the time to compile this kernel (11 to 24 s).
 constexpr int kPlanesLoad = 4;
 __device__ __forceinline__ bool takes_window(int np, int load, int kl, int ku) {
   if (np <= 3) return true;
