@@ -165,10 +165,12 @@ int dispatch_lu_cm(const double *A, int64_t n, int64_t lda, double *AB, int64_t 
  * Outputs, all in DEVICE memory: *d_kl, *d_ku (as detect_bandwidth), *d_status
  * (BANDLU_OK: factored, *d_info written by the factorisation; BANDLU_NOT_BANDED:
  * declined, AB, ipiv and *d_info untouched).  The factors are those of
- * dispatch_lu, bit for bit.  The factorisation kernels are enqueued from the
- * storage and pick their path on the device: the single-CTA windows, or, where
- * the storage admits a wider band, the multi-CTA kernel for kl <= 284; wider
- * bands are factored by a single CTA column by column.
+ * dispatch_lu, bit for bit.  The factorisation kernels are enqueued before the
+ * band is known, from the storage, and pick their path on the device: the
+ * single-CTA windows, or, for a wider band, the multi-CTA kernel where kl <= 284
+ * and that kernel can be enqueued for this ldab (its buffers hold four columns of
+ * the storage each: ldab up to about 1190).  Any other band is factored by a single
+ * CTA column by column, which is far slower: keep ldab close to 2*kl+ku+1 here.
  * Arguments: 1 A, 2 n, 3 lda, 4 AB, 5 ldab (1 <= ldab < 2^31), 6 ipiv,
  * 7 d_kl, 8 d_ku, 9 d_status, 10 d_info (DEVICE, distinct).
  * Returns BANDLU_OK (work enqueued), -i for a bad argument i, BANDLU_ERR_CUDA.

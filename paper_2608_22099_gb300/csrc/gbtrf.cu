@@ -568,9 +568,12 @@ __device__ __forceinline__ void window_factor_k(int K, int n, int kl, int ku, do
 // and the dispatch decision read from device memory.  kWinWarps warps and
 // smem_bytes of dynamic shared memory, enough for every shared-memory window
 // that fits the band storage (2*kl+ku+1 <= ldab); the block takes the path
-// launch_gbtrf would take, except that bands beyond the windows run the
-// block-wide generic elimination (the multi-CTA kernel's grid and scratch are
-// sized from kl on the host).
+// launch_gbtrf would take.  A band beyond the windows is left to the multi-CTA
+// kernel enqueued behind this one where that kernel takes it (up to wide_rows_cap
+// panel rows); else the block runs the generic elimination itself.
+// All windows share the 96 registers of 640 threads, and the widest spill (120 bytes):
+// n = 4096, us dispatch_lu / dispatch_lu_async: kl = ku = 27 2424 / 2401, kl = 27, ku = 74 3956 /
+// 4058, kl = 20, ku = 100 3598 / 3723.
 __global__ void __launch_bounds__(kWinWarps * 32, 1) k_gbtrf_on_device(int n, double *__restrict__ AB, long long ldab,
                                                                      int *__restrict__ ipiv,
                                                                      const int *__restrict__ d_kl,

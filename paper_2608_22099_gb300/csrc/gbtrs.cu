@@ -8,10 +8,11 @@
 //   backward j = n-1..0: if b_j != 0, b_j = b_j / u_jj and rows j-kv..j-1 take
 //            fma(-b_j, u, .).
 // The active part of b stays in registers (trwin.cuh): one warp per right-hand
-// side and sweep up to a window of kOneWarp rows, a CTA above.  The division by
-// u_jj uses a reciprocal formed ahead of time (div_quick).  The same operations in
-// the same order as the oracle, so the solution is bit-identical to it.  Interchanges outside j..j+kl (not produced by gbtrf)
-// are ignored.
+// side and sweep up to a window of kOneWarp rows (kOneWarpMany backward for many
+// right-hand sides), a CTA above.  The division by u_jj uses a reciprocal formed
+// ahead of time (div_quick).  The same operations in the same order as the oracle,
+// so the solution is bit-identical to it.  Interchanges outside j..j+kl (not
+// produced by gbtrf) are ignored.
 #include <algorithm>
 #include <climits>
 
