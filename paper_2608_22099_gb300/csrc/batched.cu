@@ -347,7 +347,7 @@ int launch_batched(const double *A, int64_t n, int64_t lda, int64_t strideA, int
   if (n == 0) return BANDLU_OK;
   const int wpb = 4;
   const long long grid2 = 2 * (((batch + 1) / 2 + wpb - 1) / wpb);  // two warps per pair of matrices
-  const int win_ok = (n + 1) * ldab < (int64_t)INT_MAX;  // 32-bit offsets in window_gbtrf
+  const int win_ok = ldab <= (INT_MAX - 1) / (n + 1);  // 32-bit offsets in window_gbtrf: (n + 1) * ldab < INT_MAX
   // warps to a sub-partition (every band that storage of up to seven rows admits goes in pairs)
   const long long subs = 4ll * device_sms(), load = ((ldab <= 7 ? (batch + 1) / 2 : batch) + subs - 1) / subs;
   if (load <= kPlanesLoad)

@@ -532,7 +532,9 @@ __global__ void __launch_bounds__(32) k_gbtrf_regwin(int n, int kl, int ku, doub
 }
 
 // The register window's 32-bit offsets reach every entry.
-__host__ __device__ inline bool offsets_fit(long long n, long long ldab) { return (n + 1) * ldab < (long long)INT_MAX; }
+__host__ __device__ inline bool offsets_fit(long long n, long long ldab) {
+  return ldab <= (INT_MAX - 1) / (n + 1);  // (n + 1) * ldab < INT_MAX
+}
 
 // The path choice of launch_gbtrf (without the multi-CTA kernel), shared by the
 // host launcher and the device-side dispatch: 0 register window, 1 shared-memory

@@ -191,7 +191,7 @@ int launch_block_fwd(int n, int kl, int ku, int nrhs, const double *AB, int ldab
   // us staged / from memory: kl = 100, ku = 10, 304 right-hand sides 404 / 431, 456 606 / 490, 4096 4077 /
   // 3342; kl = ku = 250, 152 416 / 443, 304 814 / 695, 4096 10690 / 9090).
   const size_t staged = 64 * (size_t)trwin::stage_pitch(kl) * sizeof(double);
-  const size_t own = staged + sizeof(trwin::Ring) + sizeof(trwin::BlockShared) + 2048;  // (and what the driver keeps)
+  const size_t own = staged + sizeof(trwin::Ring) + sizeof(trwin::BlockShared) + 2048;  // (and what CUDA keeps)
   if (kl <= trwin::kStageWidth && nrhs <= (long long)device_sms() * std::max<long long>(1, 228 * 1024 / own)) {
     constexpr int most = 64 * trwin::stage_pitch(trwin::kStageWidth) * (int)sizeof(double);
     if (!allow_dynamic_smem(reinterpret_cast<const void *>(k_gbtrs_block_fwd<512, true>), most)) return BANDLU_ERR_CUDA;

@@ -198,7 +198,7 @@ __host__ __device__ __forceinline__ double rcp_rn(double b) {
 // (mx * 2^11) * R ~ 2^62 * mx/md, short by less than 5 (three low partial products
 // are dropped) and long by less than 1.5.  It has 62 or 63 bits, so rounding it to
 // 53 is decided unless its low bits lie within that error of the rounding boundary
-// (one quotient in 100 or fewer); those, and dividends, divisors or quotients that
+// (one quotient in 64 to 128); those, and dividends, divisors or quotients that
 // are not normal numbers, take the ordinary division.  About 25 short-latency
 // instructions: on GB300 the four dependent FP64 operations of a quotient from a
 // two-term reciprocal cost 64 clk each.
