@@ -11,10 +11,10 @@
 // detection kernel reads the whole matrix and waits for that kernel to finish
 // (griddepcontrol.wait) only before its atomics, so the reset costs no gap
 // between launches.  Where the rows are contiguous (lda = 2*ceil(n/2) and A
-// 16-byte aligned), or have little padding (any address, any lda), the matrix is
-// one run of 16-byte vectors and every block reads an equal share of it; otherwise
-// work items are (row, segment) pairs, a segment blockDim.x * U consecutive
-// vectors of one row.
+// 16-byte aligned), or have little padding (any address, any lda; aligned rows from
+// n = 4500 on), the matrix is one run of 16-byte vectors and every block reads an
+// equal share of it; otherwise work items are (row, segment) pairs, a segment
+// blockDim.x * U consecutive vectors of one row.
 #include "common.cuh"
 
 namespace bandlu {
