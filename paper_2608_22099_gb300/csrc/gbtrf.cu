@@ -574,8 +574,8 @@ __device__ __forceinline__ void window_factor_k(int K, int n, int kl, int ku, do
 // kernel enqueued behind this one where that kernel takes it (up to wide_rows_cap
 // panel rows); else the block runs the generic elimination itself.
 // All windows share the 96 registers of 640 threads, and the widest spill (120 bytes):
-// n = 4096, us dispatch_lu / dispatch_lu_async: kl = ku = 27 2424 / 2401, kl = 27, ku = 74 3956 /
-// 4058, kl = 20, ku = 100 3598 / 3723.
+// n = 4096, us dispatch_lu / dispatch_lu_async: kl = ku = 16 1509 / 1406, 27 2509 / 2408, kl = 27, ku =
+// 74 4042 / 4091, kl = 20, ku = 100 3668 / 3723 (dispatch_lu's host round trip and scratch take about 90).
 __global__ void __launch_bounds__(kWinWarps * 32, 1) k_gbtrf_on_device(int n, double *__restrict__ AB, long long ldab,
                                                                      int *__restrict__ ipiv,
                                                                      const int *__restrict__ d_kl,
